@@ -546,7 +546,7 @@ ultramem_status run_tensor(ultramem_layer *L, const Dims &d, Ptrs p, cudaStream_
     *launches = d.A + 1 + score + extras;
     if (mode == kRetrieve) return ULTRAMEM_OK;
     if ((e = um::launch_gather(dd, stage_ptrs(L, p, 3), st)) != cudaSuccess) return from_cuda(e);
-    if (d.has_proj && (e = um::launch_proj_tc(dd, stage_ptrs(L, p, 4), mp, st)) != cudaSuccess)
+    if (d.has_proj && (e = um::launch_proj_tc(dd, stage_ptrs(L, p, 4), mp, 2, st)) != cudaSuccess)
         return from_cuda(e);
     *launches = d.A + 2 + score + (d.has_proj ? 1 : 0) + extras;
     if (L->profiling) L->profiled_once = true;
@@ -560,6 +560,66 @@ ultramem_status run(ultramem_layer *L, const Dims &d, Ptrs p, cudaStream_t st, R
                                     : run_cuda_core(L, d, p, st, mode, &n);
     if (s == ULTRAMEM_OK) L->launches = n;
     return s;
+}
+
+// S7-S9 on given slots (p.idx_in, p.w_in): the lookup-reduce.  With slot_pos
+// the rows were looked up elsewhere (ultramem_shard_pool): slot s reads row
+// slot_pos[s] of p.values.
+//
+// Tensor layers project on the tensor cores, with the pooled rows as three
+// bf16 terms, which carry the fp32 sums exactly, so the output is as accurate
+// as the CUDA-core projection's.  That one was the bound: 500 of 563 us at
+// the 4M-slot layer with 2048 tokens.  Measured on GB300, a call as graph
+// replays, CUDA cores -> tensor cores with the gather reading the addresses:
+// mid_4m 33.2 -> 11.3 us at 1 token, 55.5 -> 13.3 at 128, 562 -> 69 at 2048,
+// 2071 -> 272 at 8192; decode_1m 20.5 -> 8.8 at 1 token, 26.8 -> 10.1 at 64.
+// It is faster down to the smallest layers (13.3 -> 7.2 us at 2^18 multiply-
+// adds); the line at 2^19 leaves those on the four launches (slots, gather,
+// projection, reduce) that ultramem_last_launches has always reported there.
+// fp32 storage keeps the CUDA-core projection (compensated sums).
+constexpr int64_t kTcLookupMacs = 1ll << 19;
+ultramem_status pool_and_project(ultramem_layer *L, const Dims &d0, Ptrs p,
+                                 const int32_t *slot_pos, cudaStream_t st) {
+    cudaError_t e;
+    Dims d = d0;
+    int n = 0;
+    const int64_t macs = (int64_t)d.B * d.E * d.d_v * d.d_out;
+    CUtensorMap acc_map;
+    const bool tc = L->tc && d.has_proj && macs >= kTcLookupMacs &&
+                    um::tc_encode(&acc_map, L->ws.acc_bf, 3ull * d.E * d.d_v,
+                                  (uint64_t)L->cfg.max_tokens, 1, (uint32_t)d.p_ntile, 2);
+    if (tc) {
+        p.acc_bf = L->ws.acc_bf;
+        p.acc_terms = 3;
+    }
+    bool gathered = false;
+    if (tc && !slot_pos &&
+        (e = um::launch_gather_addresses(d, stage_ptrs(L, p, 3), &gathered, st)) != cudaSuccess)
+        return from_cuda(e);
+    if (gathered) {
+        n = 1;
+    } else {
+        e = slot_pos ? um::launch_shard_slots(d, p, slot_pos, st)
+                     : um::launch_slots_from_addresses(d, p, st);
+        if (e != cudaSuccess) return from_cuda(e);
+        if ((e = um::launch_gather(d, stage_ptrs(L, p, 3), st)) != cudaSuccess)
+            return from_cuda(e);
+        n = 2;
+    }
+    if (tc) {
+        um::TcMaps mp = L->maps;
+        mp.acc = acc_map;
+        d.pdl = 1;   // the projector's tiles stream in while the gather finishes
+        if ((e = um::launch_proj_tc(d, stage_ptrs(L, p, 4), mp, 3, st)) != cudaSuccess)
+            return from_cuda(e);
+        n += 1;
+    } else if (d.has_proj) {
+        if ((e = um::launch_proj(d, stage_ptrs(L, p, 4), st)) != cudaSuccess)
+            return from_cuda(e);
+        n += 2;
+    }
+    L->launches = n;
+    return ULTRAMEM_OK;
 }
 
 }  // namespace
@@ -754,8 +814,8 @@ ultramem_status ultramem_create(const ultramem_config *cfg, const ultramem_weigh
         // tensor path: split queries, bf16 acc, K-major copy of the projectors
         e = dalloc(&ws.qs, (size_t)2 * H * Bm * 3 * cfg->d_k);
         if (e == cudaSuccess) e = cudaMemset(ws.qs, 0, sizeof(__nv_bfloat16) * 2 * H * Bm * 3 * cfg->d_k);
-        if (e == cudaSuccess) e = dalloc(&ws.acc_bf, 2 * Bm * kd);   // hi, lo terms
-        if (e == cudaSuccess) e = cudaMemset(ws.acc_bf, 0, sizeof(__nv_bfloat16) * 2 * Bm * kd);
+        if (e == cudaSuccess) e = dalloc(&ws.acc_bf, 3 * Bm * kd);   // two or three terms
+        if (e == cudaSuccess) e = cudaMemset(ws.acc_bf, 0, sizeof(__nv_bfloat16) * 3 * Bm * kd);
         if (e == cudaSuccess && cfg->has_proj) {
             e = dalloc(&ws.w_pt, kd * cfg->d_out);
             if (e == cudaSuccess) e = um::launch_transpose_bf16(w->w_proj, ws.w_pt, (int)kd, cfg->d_out, 0);
@@ -905,13 +965,9 @@ ultramem_status ultramem_lookup_reduce(ultramem_layer *L, const int64_t *idx, co
     cudaError_t e;
     cudaGetLastError();
     if ((e = reset_stamps(L, st)) != cudaSuccess) return from_cuda(e);
-    if ((e = um::launch_slots_from_addresses(d, p, st)) != cudaSuccess) return from_cuda(e);
-    if ((e = um::launch_gather(d, stage_ptrs(L, p, 3), st)) != cudaSuccess) return from_cuda(e);
-    if (d.has_proj && (e = um::launch_proj(d, stage_ptrs(L, p, 4), st)) != cudaSuccess)
-        return from_cuda(e);
-    L->launches = 2 + (d.has_proj ? 2 : 0);
-    if (L->profiling) L->profiled_once = true;
-    return ULTRAMEM_OK;
+    const ultramem_status s = pool_and_project(L, d, p, nullptr, st);
+    if (s == ULTRAMEM_OK && L->profiling) L->profiled_once = true;
+    return s;
 }
 
 ultramem_status ultramem_lookup_reduce_backward(ultramem_layer *L, const int64_t *idx,
@@ -1126,13 +1182,8 @@ ultramem_status ultramem_shard_pool(ultramem_layer *L, const int64_t *idx, const
     p.out = out;
     p.values = back_rows;   // slot s reads returned row slot_pos[s]
     cudaStream_t st = (cudaStream_t)stream;
-    cudaError_t e;
     cudaGetLastError();
-    if ((e = um::launch_shard_slots(d, p, slot_pos, st)) != cudaSuccess) return from_cuda(e);
-    if ((e = um::launch_gather(d, p, st)) != cudaSuccess) return from_cuda(e);
-    if (d.has_proj && (e = um::launch_proj(d, p, st)) != cudaSuccess) return from_cuda(e);
-    L->launches = 2 + (d.has_proj ? 2 : 0);
-    return ULTRAMEM_OK;
+    return pool_and_project(L, d, p, slot_pos, st);
 }
 
 ultramem_status ultramem_debug_wait_probe(ultramem_layer *L) {

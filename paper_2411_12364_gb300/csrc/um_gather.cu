@@ -187,7 +187,11 @@ size_t bucket_smem_bytes(const Dims &d, int warps) {
 // grids, where CTAs in their bucketing or reduction phase overlap others'
 // loads (measured: 6.5 TB/s over 2.15 GB at 16384 tokens, against 5.4 with
 // 512).
-template <typename T, int THREADS>
+// ADDR: the slots come as given addresses and weights (p.idx_in, p.w_in)
+// instead of the selection's sel_row / sel_p / sel_w, and each thread works
+// its slot out itself: the slots kernel before the gather, its launch and
+// the round trip of 12 bytes a slot through memory go.
+template <typename T, int THREADS, bool ADDR>
 __global__ void __launch_bounds__(THREADS, 1024 / THREADS) gather_bucket_kernel(Dims d, Ptrs p) {
     constexpr int kBThreads = THREADS, kBWarps = THREADS / 32;
     extern __shared__ __align__(16) unsigned char gsm[];
@@ -212,11 +216,17 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS) gather_bucket_kernel(
 #pragma unroll
     for (int ci = 0; ci < kMaxCores; ++ci) w[ci] = 0.f;
     if (t < hm) {
-        row = p.sel_row[base + t];
-        blk = p.sel_p[base + t];
+        bool ok = true;   // an invalid address weighs 0
+        if constexpr (ADDR) {
+            ok = slot_of_address(d, p, p.idx_in[base + t], row, blk);
+        } else {
+            row = p.sel_row[base + t];
+            blk = p.sel_p[base + t];
+        }
+        const float *ws = ADDR ? p.w_in : p.sel_w;
 #pragma unroll
         for (int ci = 0; ci < kMaxCores; ++ci)
-            if (ci < nc) w[ci] = p.sel_w[(base + t) * nc + ci];
+            if (ci < nc) w[ci] = ok ? ws[(base + t) * nc + ci] : 0.f;
         if (blk < 0 || blk >= E) blk = -1;   // not a slot of this layer: skipped
     }
     int rank = 0;
@@ -457,32 +467,52 @@ cudaError_t configure_gather(const Dims &) {
     if (e == cudaSuccess) e = allow_padded<gather_reg_kernel<__nv_bfloat16, 1>>();
     if (e == cudaSuccess) e = allow_padded<gather_reg_kernel<__nv_bfloat16, 4>>();
     // the bucketed kernels may also be padded up to a whole SM's share (spread_smem)
-    if (e == cudaSuccess) e = allow_padded<gather_bucket_kernel<float, 512>>();
-    if (e == cudaSuccess) e = allow_padded<gather_bucket_kernel<__nv_bfloat16, 512>>();
-    if (e == cudaSuccess) e = allow_padded<gather_bucket_kernel<float, 256>>();
-    if (e == cudaSuccess) e = allow_padded<gather_bucket_kernel<__nv_bfloat16, 256>>();
+    if (e == cudaSuccess) e = allow_padded<gather_bucket_kernel<float, 512, false>>();
+    if (e == cudaSuccess) e = allow_padded<gather_bucket_kernel<__nv_bfloat16, 512, false>>();
+    if (e == cudaSuccess) e = allow_padded<gather_bucket_kernel<float, 256, false>>();
+    if (e == cudaSuccess) e = allow_padded<gather_bucket_kernel<__nv_bfloat16, 256, false>>();
+    if (e == cudaSuccess) e = allow_padded<gather_bucket_kernel<__nv_bfloat16, 512, true>>();
+    if (e == cudaSuccess) e = allow_padded<gather_bucket_kernel<__nv_bfloat16, 256, true>>();
     return e;
+}
+
+// The bucketed gather, where it serves the layer's shape (*taken).
+template <typename T, bool ADDR>
+static cudaError_t launch_bucket(const Dims &d, const Ptrs &p, bool *taken, cudaStream_t st) {
+    constexpr int epv = 16 / (int)sizeof(T);
+    *taken = true;
+    if (d.d_v / epv <= 32 && d.d_v % epv == 0 && d.E <= kBMaxE) {
+        // spread over the SMs (see spread_smem)
+        if (d.B <= 2 * 152 && d.H * d.m <= 512) {
+            constexpr auto k = gather_bucket_kernel<T, 512, ADDR>;
+            return launch_kernel(d.pdl, k, d.B, 512,
+                                 spread_smem(bucket_smem_bytes(d, 16), static_smem_of<k>(), d.B),
+                                 st, d, p);
+        }
+        if (d.H * d.m <= 256 && d.E <= 8) {
+            constexpr auto k = gather_bucket_kernel<T, 256, ADDR>;
+            return launch_kernel(d.pdl, k, d.B, 256,
+                                 spread_smem(bucket_smem_bytes(d, 8), static_smem_of<k>(), d.B),
+                                 st, d, p);
+        }
+    }
+    *taken = false;
+    return cudaSuccess;
+}
+
+cudaError_t launch_gather_addresses(const Dims &d, const Ptrs &p, bool *taken, cudaStream_t st) {
+    *taken = false;
+    if (d.dtype != ULTRAMEM_BF16) return cudaSuccess;
+    return launch_bucket<__nv_bfloat16, true>(d, p, taken, st);
 }
 
 template <typename T>
 static cudaError_t launch_gather_t(const Dims &d, const Ptrs &p, cudaStream_t st) {
     const size_t bytes = gather_smem_bytes(d);
     const bool fits_lanes = d.d_v / (16 / (int)sizeof(T)) <= 32;
-    if (fits_lanes && d.d_v % (16 / (int)sizeof(T)) == 0 && d.E <= kBMaxE) {
-        // spread over the SMs (see spread_smem)
-        if (d.B <= 2 * 152 && d.H * d.m <= 512) {
-            constexpr auto k = gather_bucket_kernel<T, 512>;
-            return launch_kernel(d.pdl, k, d.B, 512,
-                                 spread_smem(bucket_smem_bytes(d, 16), static_smem_of<k>(), d.B),
-                                 st, d, p);
-        }
-        if (d.H * d.m <= 256 && d.E <= 8) {
-            constexpr auto k = gather_bucket_kernel<T, 256>;
-            return launch_kernel(d.pdl, k, d.B, 256,
-                                 spread_smem(bucket_smem_bytes(d, 8), static_smem_of<k>(), d.B),
-                                 st, d, p);
-        }
-    }
+    bool taken;
+    const cudaError_t be = launch_bucket<T, false>(d, p, &taken, st);
+    if (taken) return be;
     // the shared-memory-accumulating kernel: fp64 accumulators (fp32 storage)
     // while they fit, else fp32 ones
     auto general = [&]() {

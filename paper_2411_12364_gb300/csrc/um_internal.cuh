@@ -12,8 +12,9 @@
 //                                      one per value slice, Multi-Core Scoring)
 //   acc      [B][E*D_v]                per-block pooled rows, Eq. 15 inner sum
 //   acc_bf   [B][T][E*D_v] bf16        the same as T bf16 terms (tensor path):
-//                                      T = 2 for the projection, whose B operand
-//                                      is then hi + lo (residual <= 2^-16 |acc|)
+//                                      T = 2 for the forward's projection, whose B
+//                                      operand is then hi + lo (residual <= 2^-16
+//                                      |acc|); T = 3 for the lookup-reduce's (exact)
 //   proj_part[p_splits][B][D'_v]       split-K partial sums of the projection
 //   xs       the convolved query input x~ (Trick 4): bf16 [B][3][D_i], three
 //            terms per value, for the tensor-core query; fp32 [B][D_i] for
@@ -84,7 +85,8 @@ struct Ptrs {
     float *w_out;
     __nv_bfloat16 *acc_bf;       // tensor path: acc as bf16 terms [B][acc_terms][E*D_v]
     int acc_terms;               // 2: hi + lo, the pooled value to 2^-16 relative (the
-                                 // projection's operand); 1 (or 0): one rounding
+                                 // forward's projection); 3: hi + mid + lo, the pooled
+                                 // value exactly (the lookup-reduce's)
     const int64_t *idx_in;       // lookup_reduce input addresses
     const float *w_in;           // lookup_reduce input weights [B][H][m][nc]
     const float *conv_w, *conv_b;   // [conv_k][D_i], [D_i] or null
@@ -124,7 +126,9 @@ cudaError_t configure_small();
 // instead of x itself
 cudaError_t launch_query_small(const Dims &d, const Ptrs &p, __nv_bfloat16 *qs, int Bmax,
                                bool x_f32, bool write_qs, bool pdl, cudaStream_t st);
-cudaError_t launch_proj_tc(const Dims &d, const Ptrs &p, const TcMaps &mp, cudaStream_t st);
+// acc_terms: bf16 terms of the pooled rows (map acc over [B][acc_terms E D_v])
+cudaError_t launch_proj_tc(const Dims &d, const Ptrs &p, const TcMaps &mp, int acc_terms,
+                           cudaStream_t st);
 // the backward's dacc = W_p g on the tensor cores (g: map over [B][D'_v] bf16)
 cudaError_t launch_dacc_tc(const Dims &d, const CUtensorMap &w_p, const CUtensorMap &g,
                            float *dacc, int *err, cudaStream_t st);
@@ -154,6 +158,10 @@ cudaError_t launch_score(const Dims &d, const Ptrs &p, cudaStream_t st);
 cudaError_t launch_select(const Dims &d, const Ptrs &p, cudaStream_t st);
 cudaError_t launch_slots_from_addresses(const Dims &d, const Ptrs &p, cudaStream_t st);
 cudaError_t launch_gather(const Dims &d, const Ptrs &p, cudaStream_t st);
+// The gather of given addresses (p.idx_in, p.w_in), without a slots kernel
+// before it; *taken = false (and nothing launched) for the shapes that only
+// the kernels reading sel_row / sel_p / sel_w serve.
+cudaError_t launch_gather_addresses(const Dims &d, const Ptrs &p, bool *taken, cudaStream_t st);
 cudaError_t launch_proj(const Dims &d, const Ptrs &p, cudaStream_t st);
 
 // The number-wise partitioned table (App. D): route slots to their rows'
@@ -359,19 +367,36 @@ __device__ __forceinline__ void put_split_query(__nv_bfloat16 *qs, int axis, int
     dst[2 * d_k] = q3;
 }
 
+// v with its low 16 bits cleared: the bf16 next to v towards zero.
+__device__ __forceinline__ float cut_bf16(float v) {
+    return __uint_as_float(__float_as_uint(v) & 0xffff0000u);
+}
+
 // One pooled value acc[b][i] (i < E*D_v) into the buffer the next step
-// reads: the tensor path's bf16 terms (hi = rn(v), lo = rn(v - hi), so that
-// hi + lo equals v to 2^-16 relative), the fp32 acc of the CUDA-core
-// projection, or, without a projector, the output row itself.
+// reads: the tensor path's bf16 terms, the fp32 acc of the CUDA-core
+// projection, or, without a projector, the output row itself.  Two terms:
+// hi = rn(v), lo = rn(v - hi), so that hi + lo equals v to 2^-16 relative.
+// Three terms: v cut (not rounded) into its leading 8 significant bits, the
+// next 8 and the last 8, whose sum is v exactly (down to the subnormals); a
+// value that is not finite stays in the first term alone.
 template <typename T>
 __device__ __forceinline__ void store_pooled(const Dims &d, const Ptrs &p, int64_t b, int i,
                                              float v) {
     const int EDv = d.E * d.d_v;
     if (p.acc_bf) {
-        const __nv_bfloat16 hi = __float2bfloat16_rn(v);
-        __nv_bfloat16 *dst = p.acc_bf + b * (p.acc_terms > 1 ? 2 : 1) * EDv + i;
-        dst[0] = hi;
-        if (p.acc_terms > 1) dst[EDv] = __float2bfloat16_rn(v - __bfloat162float(hi));
+        __nv_bfloat16 *dst = p.acc_bf + b * p.acc_terms * EDv + i;
+        if (p.acc_terms == 3) {
+            const bool fin = fabsf(v) < __int_as_float(0x7f800000);
+            const float hi = fin ? cut_bf16(v) : v, r1 = fin ? v - hi : 0.f;
+            const float mid = cut_bf16(r1);
+            dst[0] = __float2bfloat16_rn(hi);
+            dst[EDv] = __float2bfloat16_rn(mid);
+            dst[2 * EDv] = __float2bfloat16_rn(r1 - mid);
+        } else {
+            const __nv_bfloat16 hi = __float2bfloat16_rn(v);
+            dst[0] = hi;
+            dst[EDv] = __float2bfloat16_rn(v - __bfloat162float(hi));
+        }
     } else if (d.has_proj) {
         p.acc[b * EDv + i] = v;
     } else {
@@ -429,6 +454,23 @@ __device__ __forceinline__ uint64_t shuffle_address(const Dims &d, const uint32_
     if (r >= d.M) r -= d.M;
     if (r >= d.M) r -= d.M;
     return r;
+}
+
+// A given virtual address as its block and physical row; an address outside
+// [0, E*N) is recorded in the error word and read as address 0 (the caller
+// gives it weight 0).  Returns whether the address is valid.
+__device__ __forceinline__ bool slot_of_address(const Dims &d, const Ptrs &p, int64_t v, int &row,
+                                                int &blk) {
+    const bool ok = v >= 0 && (uint64_t)v < d.M;
+    if (!ok) {
+        atomicOr(p.err, kErrBadIndex);
+        v = 0;
+    }
+    const uint32_t vs = (uint32_t)shuffle_address(d, p.perm, (uint64_t)v);   // < M < 2^32
+    const uint32_t N = (uint32_t)d.N, pb = vs / N;
+    row = (int)(vs - pb * N);
+    blk = (int)pb;
+    return ok;
 }
 
 }  // namespace um

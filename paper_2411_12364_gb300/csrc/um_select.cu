@@ -1331,18 +1331,12 @@ __global__ void slots_kernel(Dims d, Ptrs p) {
     const int64_t total = (int64_t)d.B * d.H * d.m;
     for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < total;
          e += (int64_t)gridDim.x * blockDim.x) {
-        int64_t v = p.idx_in[e];
-        const bool bad = v < 0 || (uint64_t)v >= d.M;
-        if (bad) {
-            atomicOr(p.err, kErrBadIndex);
-            v = 0;
-        }
+        int row, blk;
+        const bool ok = slot_of_address(d, p, p.idx_in[e], row, blk);
         for (int ci = 0; ci < d.nc; ++ci)
-            p.sel_w[e * d.nc + ci] = bad ? 0.f : p.w_in[e * d.nc + ci];
-        uint64_t vs = shuffle_address(d, p.perm, (uint64_t)v);
-        uint64_t pb = vs / (uint64_t)d.N;
-        p.sel_row[e] = (int32_t)(vs - pb * (uint64_t)d.N);
-        p.sel_p[e] = (int32_t)pb;
+            p.sel_w[e * d.nc + ci] = ok ? p.w_in[e * d.nc + ci] : 0.f;
+        p.sel_row[e] = row;
+        p.sel_p[e] = blk;
     }
 }
 

@@ -1151,6 +1151,7 @@ cudaError_t configure_tc() {
     if (e == cudaSuccess) e = allow_smem<3, ScoreListOp<kListGroupMax>>();
     if (e == cudaSuccess) e = allow_smem<3, ScoreListOp<kListCandidates>>();
     if (e == cudaSuccess) e = allow_smem<2, ProjOp>();
+    if (e == cudaSuccess) e = allow_smem<3, ProjOp>();
     if (e == cudaSuccess) e = allow_smem<1, DaccOp>();
     if (e == cudaSuccess) e = allow_smem<2, DwOp>();
     return e;
@@ -1288,16 +1289,18 @@ cudaError_t launch_score_tc(const Dims &d, const Ptrs &p, const TcMaps &mp, cuda
     return launch_score_keys(d, p, mp, d.probe_wait, st);
 }
 
-cudaError_t launch_proj_tc(const Dims &d, const Ptrs &p, const TcMaps &mp, cudaStream_t st) {
+cudaError_t launch_proj_tc(const Dims &d, const Ptrs &p, const TcMaps &mp, int acc_terms,
+                           cudaStream_t st) {
     if (d.p_splits > kMaxSplits) return cudaErrorInvalidValue;
     ProjOp op;
     op.stamp = p.stamp;
     op.n_tile = d.p_ntile ? d.p_ntile : tc_n_tile(d.B, 1);
     op.n_acc = 1;
     op.acc_chunk = 1 << 30;
-    // the pooled rows are two bf16 terms hi + lo ([B][2][E D_v]): both
+    // the pooled rows are two or three bf16 terms ([B][terms][E D_v]): all
     // multiply each projector tile into one fp32 accumulator, so the operand
-    // carries the pooled value to 2^-16 relative instead of one rounding
+    // carries the pooled value to 2^-16 relative (two) or exactly (three)
+    // instead of one rounding
     op.b_split_stride = d.E * d.d_v;
     op.err = p.err;
     op.B = d.B;
@@ -1307,7 +1310,8 @@ cudaError_t launch_proj_tc(const Dims &d, const Ptrs &p, const TcMaps &mp, cudaS
     op.out = static_cast<__nv_bfloat16 *>(p.out);
     dim3 grid((d.d_out + kTileM - 1) / kTileM, (d.B + op.n_tile - 1) / op.n_tile, op.splits);
     const int per = (op.kb_total + op.splits - 1) / op.splits;
-    return launch_gemm<2>(grid, mp.w_pt, mp.w_pt, mp.acc, op, per, d.pdl, st);
+    return acc_terms == 3 ? launch_gemm<3>(grid, mp.w_pt, mp.w_pt, mp.acc, op, per, d.pdl, st)
+                          : launch_gemm<2>(grid, mp.w_pt, mp.w_pt, mp.acc, op, per, d.pdl, st);
 }
 
 }  // namespace um
