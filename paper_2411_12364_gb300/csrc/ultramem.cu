@@ -455,9 +455,10 @@ ultramem_status run_cuda_core(ultramem_layer *L, const Dims &d0, Ptrs p, cudaStr
         d.q_splits = 1;   // the normalised query is split 0
     }
     if (mode == kExact) {
-        if ((e = um::launch_exact(d, p, p.idx_out, p.w_out, st)) != cudaSuccess)
+        int n = 0;
+        if ((e = um::launch_exact(d, p, p.idx_out, p.w_out, &n, st)) != cudaSuccess)
             return from_cuda(e);
-        *launches = 2 + extras;
+        *launches = 1 + n + extras;
         return ULTRAMEM_OK;
     }
     if ((e = um::launch_score(d, stage_ptrs(L, p, 1), st)) != cudaSuccess) return from_cuda(e);
@@ -530,9 +531,10 @@ ultramem_status run_tensor(ultramem_layer *L, const Dims &d, Ptrs p, cudaStream_
     if (mode == kExact) {
         Dims dx = dd;
         dx.q_splits = 1;   // the summed query is split 0
-        if ((e = um::launch_exact(dx, p, p.idx_out, p.w_out, st)) != cudaSuccess)
+        int n = 0;
+        if ((e = um::launch_exact(dx, p, p.idx_out, p.w_out, &n, st)) != cudaSuccess)
             return from_cuda(e);
-        *launches = d.A + 1 + extras;
+        *launches = d.A + n + extras;
         return ULTRAMEM_OK;
     }
     if ((e = um::launch_score_tc(dd, stage_ptrs(L, p, 1), mp, st)) != cudaSuccess)

@@ -177,11 +177,12 @@ cudaError_t launch_shard_slots(const Dims &d, const Ptrs &p, const int32_t *slot
                                cudaStream_t st);
 
 // Eq. 5 by brute force (recall measurement): the exact top-m of every
-// (token, head)'s whole grid into idx_out / w_out [B][H][m]
+// (token, head)'s whole grid into idx_out / w_out [B][H][m]; *launches: the
+// kernels launched
 bool exact_fits(const Dims &d);
 cudaError_t configure_exact(const Dims &d);
 cudaError_t launch_exact(const Dims &d, const Ptrs &p, int64_t *idx_out, float *w_out,
-                         cudaStream_t st);
+                         int *launches, cudaStream_t st);
 
 // The backward of the lookup-reduce (App. D): dacc = W_p g, then dV (+=) and
 // dw from the slots (p.idx_in, p.w_in); dW_p from the forward's pooled rows
