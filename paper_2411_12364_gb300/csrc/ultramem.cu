@@ -22,7 +22,7 @@ const char *const kStageNames[kStages] = {"query", "score", "select", "gather", 
 struct Workspace {
     float *q_part = nullptr, *sel_w = nullptr, *acc = nullptr, *proj_part = nullptr;
     uint32_t *akey = nullptr;   // the rank-1 keys [B][H][2][K], or (Dims::cand) the
-                                // candidate lists [B][H][2][16 G] u64 in the same space
+                                // candidate lists [B][H][2][64 n_segs] u64 in the same space
     uint32_t *gstat = nullptr, *tau = nullptr;   // candidate lists: group maxima / counts, bounds
     int32_t *sel_row = nullptr, *sel_p = nullptr;
     float *core = nullptr, *u = nullptr, *t = nullptr;
@@ -729,6 +729,7 @@ ultramem_status ultramem_create(const ultramem_config *cfg, const ultramem_weigh
     d.dk = cfg->d_k / r;
     d.K = (int)keys_per_axis(*cfg);
     d.n_groups = (d.K + 15) / 16;
+    d.n_segs = (d.K + 63) / 64;
     d.N = (int64_t)cfg->n * cfg->n;
     d.M = (uint64_t)cfg->expand_e * (uint64_t)d.N;
     d.E = cfg->expand_e;
@@ -773,11 +774,11 @@ ultramem_status ultramem_create(const ultramem_config *cfg, const ultramem_weigh
     const size_t hm = Bm * H * cfg->topm;
     if (e == cudaSuccess) e = dalloc(&ws.q_part, qmax * d.A * HD);
     // the candidate-list scoring (long grids, tensor path) keeps its u64
-    // lists (16 G entries an axis) where the keys would be
+    // lists (64 entries per 64 keys of an axis) where the keys would be
     L->cand_ok = L->tc && d.n_groups >= d.k && d.n_groups <= 1024;
     const size_t lists = Bm * H * 2;
     const size_t key_words = lists * (size_t)d.K;
-    const size_t list_words = lists * 16 * (size_t)d.n_groups * 2;
+    const size_t list_words = lists * 64 * (size_t)d.n_segs * 2;
     if (e == cudaSuccess)
         e = dalloc(&ws.akey, L->cand_ok && list_words > key_words ? list_words : key_words);
     if (e == cudaSuccess && L->cand_ok) e = dalloc(&ws.gstat, lists * (size_t)d.n_groups);

@@ -64,6 +64,7 @@ struct Dims {
     int cand;          // tensor path, long grids: the scoring leaves per-axis
                        // candidate lists instead of every key (see ScoreOp)
     int n_groups;      // candidate lists: groups of 16 keys an axis, ceil(K / 16)
+    int n_segs;        // and segments of 64 keys, ceil(K / 64)
 };
 
 struct Ptrs {
@@ -74,9 +75,10 @@ struct Ptrs {
     float *q_part, *sel_w, *acc, *proj_part;
     uint32_t *akey;
     // candidate lists (Dims::cand): per (token, head, axis) the largest key
-    // of each group of 16 keys, then the group's count of candidates
-    // [B][H][2][n_groups], the bound tau [B][H][2] and the list of
-    // composites, a 16-entry segment per group [B][H][2][n_groups][16]
+    // of each group of 16 keys [B][H][2][n_groups], then (in the same space)
+    // the count of candidates of each segment of 64 keys [B][H][2][n_segs],
+    // the bound tau [B][H][2] and the list of composites, a 64-entry segment
+    // per 64 keys [B][H][2][n_segs][64]
     uint32_t *gstat, *tau;
     unsigned long long *cand;
     int32_t *sel_row, *sel_p;
@@ -338,6 +340,35 @@ __device__ __forceinline__ uint32_t f2ord(float f) {
 __device__ __forceinline__ float ord2f(uint32_t o) {
     uint32_t u = (o & 0x80000000u) ? (o & 0x7fffffffu) : ~o;
     return __uint_as_float(u);
+}
+
+// Two fp32 values in a 64-bit register; the packed instructions round each
+// half as the scalar ones do.
+typedef unsigned long long f2;
+__device__ __forceinline__ f2 pack2(float a, float b) {
+    f2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+    return r;
+}
+__device__ __forceinline__ float2 unpack2(f2 v) {
+    float2 r;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
+    return r;
+}
+__device__ __forceinline__ f2 mul2(f2 a, f2 b) {
+    f2 r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ f2 fma2(f2 a, f2 b, f2 c) {
+    f2 r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+__device__ __forceinline__ f2 add2(f2 a, f2 b) {
+    f2 r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
 }
 
 // A selection candidate: (key, position) as one 64-bit value whose

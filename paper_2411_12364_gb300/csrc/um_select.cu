@@ -256,15 +256,14 @@ __device__ __forceinline__ void warp_append(bool pr, u64 comp, u64 *list, int *c
 
 // The scoring's candidate list of axis s (Dims::cand): every key of the
 // axis' top k is in it, with the keys above a bound, as composites.  The
-// list is G segments of 16 entries (one per group of 16 keys); segment g
-// holds its group's candidates in its first cnt[g] entries (the counts
-// replace the group maxima in gstat).  Up to kCap entries are gathered
-// into cand[s] (placed by a block scan of the threads' counts); a longer
-// list (heavy ties) is replaced by its exact top kk, a radix select over the
-// 64-bit composites (distinct: exactly kk are >= the kk-th largest).
-// Length in cnt[slot].  Whole block; ends with a barrier.
-constexpr int kSeg = 16;               // entries of a list segment (keys of a group)
-constexpr int kMaxSegPerThread = 4;   // G <= 1024 segments
+// list is G segments of 64 entries (one per 64 keys); segment g holds its
+// keys' candidates, in position order, in its first cnt[g] entries.  Up to
+// kCap entries are gathered into cand[s] (placed by a block scan of the
+// threads' counts); a longer list (heavy ties) is replaced by its exact top
+// kk, a radix select over the 64-bit composites (distinct: exactly kk are >=
+// the kk-th largest).  Length in cnt[slot].  Whole block; ends with a barrier.
+constexpr int kSeg = 64;               // keys and entries of a list segment
+constexpr int kMaxSegPerThread = 1;   // G <= 256 segments
 __device__ __noinline__ void cand_fallback(const u64 *seg, const uint32_t *cnt, int G, int kk,
                                            int s, int slot, SelShared &sh) {
     const int n = kSeg * G;
@@ -301,7 +300,7 @@ __device__ __noinline__ void cand_fallback(const u64 *seg, const uint32_t *cnt, 
 // Both axes' lists of one (token, head) (lists `list0` and `list0 + 1`)
 // into cand[0] and cand[1], lengths in cnt[kCntAxis + s].  One block scan
 // places both (the two axes' counts packed in the low and high 16 bits:
-// each total is at most 16 G <= 16384), and each thread loads the first
+// each total is at most 64 G <= 16384), and each thread loads the first
 // entry of all its segments before it stores any, so that the copies cost
 // one round trip to memory, not one per segment.  Whole block; ends with a
 // barrier.
@@ -683,14 +682,30 @@ __device__ __forceinline__ void load_keys(const uint32_t *A0, const uint32_t *A1
 
 // A 16-byte load of a key row with the L2 evict-last policy: the rows are
 // read again by the other (token, head) pairs of the batch.
-__device__ __forceinline__ uint4 ld_key_row(const uint4 *ptr) {
+__device__ __forceinline__ uint64_t key_row_policy() {
     uint64_t pol;
     asm volatile("createpolicy.fractional.L2::evict_last.b64 %0, 1.0;" : "=l"(pol));
+    return pol;
+}
+__device__ __forceinline__ uint4 ld_key_row(const uint4 *ptr, uint64_t pol) {
     uint4 v;
     asm volatile("ld.global.nc.L2::cache_hint.v4.u32 {%0, %1, %2, %3}, [%4], %5;"
                  : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
                  : "l"(ptr), "l"(pol));
     return v;
+}
+__device__ __forceinline__ uint4 ld_key_row(const uint4 *ptr) {
+    return ld_key_row(ptr, key_row_policy());
+}
+// The same into v when `go`, without a branch (which would keep the work
+// around it from interleaving).
+__device__ __forceinline__ void ld_key_row_if(uint4 &v, const uint4 *ptr, uint64_t pol, bool go) {
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "setp.ne.b32 p, %6, 0;\n\t"
+        "@p ld.global.nc.L2::cache_hint.v4.u32 {%0, %1, %2, %3}, [%4], %5;\n\t}"
+        : "+r"(v.x), "+r"(v.y), "+r"(v.z), "+r"(v.w)
+        : "l"(ptr), "l"(pol), "r"((int)go));
 }
 
 // The paired decode selection's cluster barrier (arrive, then wait).
@@ -947,11 +962,12 @@ __device__ void axis_survivors(const Dims &d, const Ptrs &p, int h, const SelLay
 // and S_col) into the row CTA's shared memory with asynchronous stores that
 // complete bytes of the row CTA's exchange mbarrier, and the row CTA, once
 // that barrier completes, goes on alone (Tucker scores, top-m, outputs).
-template <typename T, int MINB, int RM, bool PAIR = false>
-__global__ void __launch_bounds__(kThreads, MINB) select_kernel(Dims d, Ptrs p) {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    __shared__ SelShared sh;
-    const int b = blockIdx.x / d.H, h = blockIdx.x % d.H;
+// FIRST: the body of a kernel, with its dependency wait and stamps; else a
+// (token, head) that the warp-wise selection below left to its block.
+template <typename T, int MINB, int RM, bool PAIR, bool FIRST>
+__device__ __forceinline__ void select_block(const Dims &d, const Ptrs &p, int bh,
+                                             unsigned char *smem_raw, SelShared &sh) {
+    const int b = bh / d.H, h = bh % d.H;
     const int ax = PAIR ? (int)blockIdx.z : 0;   // the cluster's rank (cluster 1 x 1 x 2)
     const SelLayout L = carve(d, smem_raw);
     const int r = d.r, K = d.K, k = d.k, m = d.m;
@@ -975,9 +991,11 @@ __global__ void __launch_bounds__(kThreads, MINB) select_kernel(Dims d, Ptrs p) 
     const float *cp = p.cores + (int64_t)h * ncrr;
     const float cp0 = threadIdx.x < ncrr ? cp[threadIdx.x] : 0.f;
     const float cp1 = threadIdx.x + kThreads < ncrr ? cp[threadIdx.x + kThreads] : 0.f;
-    pdl_wait();
-    stamp_begin(p.stamp);
-    pdl_trigger();
+    if constexpr (FIRST) {
+        pdl_wait();
+        stamp_begin(p.stamp);
+        pdl_trigger();
+    }
     const int HD = d.H * d.d_k;
     const int64_t split_stride = (int64_t)d.A * d.B * HD;
     auto q_src = [&](int e) {
@@ -1026,7 +1044,7 @@ __global__ void __launch_bounds__(kThreads, MINB) select_kernel(Dims d, Ptrs p) 
         __syncthreads();
     } else if (lists) {   // the scoring left each axis' candidates
         __syncthreads();
-        load_lists(p, ((int64_t)b * d.H + h) * 2, d.n_groups, k, sh);
+        load_lists(p, ((int64_t)b * d.H + h) * 2, d.n_segs, k, sh);
     } else {
         warp_bounds(top[0][0], top[0][1], top[1][0], top[1][1], 2, k, sh);
         __syncthreads();
@@ -1280,8 +1298,840 @@ __global__ void __launch_bounds__(kThreads, MINB) select_kernel(Dims d, Ptrs p) 
                         row_bytes);
         }
     }
+    if constexpr (FIRST) stamp_end(p.stamp);
+}
+
+template <typename T, int MINB, int RM, bool PAIR = false>
+__global__ void __launch_bounds__(kThreads, MINB) select_kernel(Dims d, Ptrs p) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    __shared__ SelShared sh;
+    select_block<T, MINB, RM, PAIR, true>(d, p, (int)blockIdx.x, smem_raw, sh);
+}
+
+// ---- long grids: one warp per (token, head) ---------------------------------
+// A block per (token, head) spends most of its instructions on what a block
+// needs to work on one selection: barriers, block scans, bounds per warp,
+// and sorts of runs of 32 that are merged by searches (21.6 thousand warp
+// instructions a selection at prefill_16k, issue-bound at 2.7 a cycle).  Here
+// each of a CTA's 8 warps selects for its own (token, head), without a
+// barrier:
+//   * an axis' top k: from the candidate lists (loaded in position order), or
+//     from every key (read twice, 16 bytes a lane, with the bound taken from
+//     256 group maxima); the k-th largest key is found bit by bit over the
+//     candidates' keys in registers, from the first bit in which they differ
+//     until exactly k are at or above it;
+//   * the survivors' chunk scores, 16 (k = 64) to 8 (k = 32) rows at a time,
+//     each by the same lanes in the same order as the block does;
+//   * the k x k Tucker scores twice: a lane holds two columns and streams the
+//     rows, two at a time (packed fp32), first for 8 group maxima a lane, of
+//     which the m-th largest is the bound, then for a mask of the pairs at or
+//     above it.  Nothing of the k x k grid is stored;
+//   * the top m of those (about 120 at k = m = 64) by the same bit search,
+//     then one bitonic sort of 64 in registers.
+// The scores, the order and so the selection are those of select_block, bit
+// for bit.  What a warp cannot hold (longer lists than kWCap or kWTop, scores
+// that are not finite, a list shorter than k) it leaves to select_block: its
+// CTA takes those (token, head)s one by one after its warps are done.
+// About 7100 warp instructions a selection at prefill_16k.  Measured on GB300:
+// the selection of prefill_16k 1660 -> 620 us (a pass 2930 -> 1902), at mid_4m with
+// 1000 tokens and two cores 118 -> 64 us, at decode_1m with 2000 tokens (every
+// key) 105 -> 59 us.  Bound by latency: 8 warps a scheduler (64 registers),
+// chains of shared-memory reads, shuffles and warp reductions.
+constexpr int kWCap = 192;    // candidates of an axis
+constexpr int kWTop = 384;    // candidates of the final top m
+constexpr int kWParts = 8;    // group maxima a lane
+constexpr int kWMaxK = 64;
+constexpr int kWMaxD = 256;   // D_k
+
+// The kk-th largest of the warp's keys (key[q] of the valid entries; 0 where
+// there is none, below every key), or any value between it and the next
+// smaller one; *cnt = how many keys are at or above it (kk unless keys tie
+// with it).  1 <= kk <= c, the number of valid entries.  With a slack the
+// search stops at a value that kk to kk + slack keys reach.
+template <int NQ>
+__device__ __forceinline__ uint32_t warp_kth(const uint32_t (&key)[NQ], int c, int kk, int *cnt,
+                                             int slack = 0) {
+    uint32_t mx = 0u, mn = 0xffffffffu;
+#pragma unroll
+    for (int q = 0; q < NQ; ++q) {
+        mx = max(mx, key[q]);
+        mn = min(mn, key[q] - 1u);   // an empty entry wraps to the largest value
+    }
+    mx = __reduce_max_sync(kFull, mx);
+    mn = __reduce_min_sync(kFull, mn) + 1u;
+    *cnt = c;
+    if (c <= kk + slack || mx == mn) return mn;
+    int bit = 31 - __clz(mx ^ mn);
+    uint32_t T = mx & ~((2u << bit) - 1u);
+    for (; bit >= 0; --bit) {
+        const uint32_t t = T | (1u << bit);
+        int n = 0;
+#pragma unroll
+        for (int q = 0; q < NQ; ++q) n += key[q] >= t;
+        n = __reduce_add_sync(kFull, n);
+        if (n >= kk) {
+            T = t;
+            *cnt = n;
+            if (n <= kk + slack) break;
+        }
+    }
+    return T;
+}
+
+// put(i, entry) for the kk largest of the c <= 32 NQ composites of list
+// (distinct), i counting them in list order.
+template <int NQ, class Put>
+__device__ __forceinline__ void warp_top(const u64 *list, int c, int kk, Put put) {
+    const int lane = threadIdx.x & 31;
+    const unsigned lt = (1u << lane) - 1u;
+    uint32_t key[NQ];
+#pragma unroll
+    for (int q = 0; q < NQ; ++q) key[q] = lane + 32 * q < c ? key_of(list[lane + 32 * q]) : 0u;
+    int cnt;
+    const uint32_t T = warp_kth<NQ>(key, c, kk, &cnt);
+    unsigned win = 0u;   // bit q: this lane's entry q is taken
+#pragma unroll
+    for (int q = 0; q < NQ; ++q) win |= (uint32_t)(key[q] >= T && key[q]) << q;
+    if (cnt > kk) {   // keys tie with the kk-th: the smaller positions go first
+        unsigned tie = 0u;
+#pragma unroll
+        for (int q = 0; q < NQ; ++q) tie |= (uint32_t)(key[q] == T && key[q]) << q;
+        win &= ~tie;
+        int need = kk - (int)__reduce_add_sync(kFull, __popc(win));
+        while (need > 0) {
+            uint32_t best = 0u;   // the largest ~position of this lane's ties
+            int bq = 0;
+#pragma unroll 1
+            for (unsigned t = tie; t; t &= t - 1u) {
+                const int q = __ffs(t) - 1;
+                const uint32_t lo = (uint32_t)list[lane + 32 * q];
+                if (lo >= best) {
+                    best = lo;
+                    bq = q;
+                }
+            }
+            const uint32_t all = __reduce_max_sync(kFull, tie ? best : 0u);
+            const unsigned bal = __ballot_sync(kFull, tie && best == all);
+            if (bal == 0u) break;   // (positions are distinct: never expected)
+            if (lane == __ffs(bal) - 1) {
+                win |= 1u << bq;
+                tie &= ~(1u << bq);
+            }
+            --need;
+        }
+    }
+    int base = 0;
+#pragma unroll
+    for (int q = 0; q < NQ; ++q) {
+        const unsigned bal = __ballot_sync(kFull, (win >> q) & 1u);
+        if ((win >> q) & 1u) put(base + __popc(bal & lt), list[lane + 32 * q]);
+        base += __popc(bal);
+    }
+}
+
+// Inclusive scan over the warp.
+__device__ __forceinline__ int warp_scan(int v) {
+    const int lane = threadIdx.x & 31;
+#pragma unroll
+    for (int off = 1; off < 32; off <<= 1) {
+        const int y = __shfl_up_sync(kFull, v, off);
+        if (lane >= off) v += y;
+    }
+    return v;
+}
+
+// Both axes' candidate lists (see load_lists; counts cnt and segments seg of
+// axis 0, then of axis 1) into list0 and list1, in position order; returns
+// whether both fit kWCap, their lengths in c.  Two rounds of 32 segments, a
+// lane each, of both axes are taken together, with the loads of their counts
+// and then of their first four entries in flight at once.
+__device__ __forceinline__ bool warp_load_lists(const uint32_t *cnt, const u64 *seg, int G,
+                                                u64 *list0, u64 *list1, int (&c)[2]) {
+    const int lane = threadIdx.x & 31;
+    int total = 0;   // both lists' lengths, 16 bits each
+    for (int g0 = 0; g0 < G; g0 += 64) {
+        uint32_t n[2][2];
+        ulonglong2 e01[2][2], e23[2][2];
+#pragma unroll
+        for (int u = 0; u < 2; ++u)
+#pragma unroll
+            for (int s = 0; s < 2; ++s) {
+                const int g = g0 + 32 * u + lane;
+                n[u][s] = g < G ? min(__ldcs(cnt + s * G + g), (uint32_t)kSeg) : 0u;
+            }
+#pragma unroll
+        for (int u = 0; u < 2; ++u)
+#pragma unroll
+            for (int s = 0; s < 2; ++s) {
+                const ulonglong2 *src = reinterpret_cast<const ulonglong2 *>(
+                    seg + (int64_t)(s * G + g0 + 32 * u + lane) * kSeg);
+                if (n[u][s] > 0) e01[u][s] = __ldcs(src);
+                if (n[u][s] > 2) e23[u][s] = __ldcs(src + 1);
+            }
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+            const int both = (int)(n[u][0] | n[u][1] << 16);
+            const int incl = warp_scan(both);
+            const int before = total + incl - both;
+            total += __shfl_sync(kFull, incl, 31);
+            if ((total & 0xffff) > kWCap || (total >> 16) > kWCap) return false;   // uniform
+#pragma unroll
+            for (int s = 0; s < 2; ++s) {
+                u64 *dst = (s ? list1 : list0) + (s ? before >> 16 : before & 0xffff);
+                const uint32_t m = n[u][s];
+                if (m > 0) dst[0] = e01[u][s].x;
+                if (m > 1) dst[1] = e01[u][s].y;
+                if (m > 2) dst[2] = e23[u][s].x;
+                if (m > 3) dst[3] = e23[u][s].y;
+                const u64 *src = seg + (int64_t)(s * G + g0 + 32 * u + lane) * kSeg;
+                for (uint32_t f = 4; f < m; ++f) dst[f] = __ldcs(src + f);
+            }
+        }
+    }
+    c[0] = total & 0xffff;
+    c[1] = total >> 16;
+    return true;
+}
+
+// One axis' candidates from every key (K % 4 == 0): those at or above a
+// bound that at least kk keys reach, into list (in no order); returns their
+// number, or -1 when it is larger than kWCap.
+__device__ __forceinline__ int warp_scan_keys(const uint32_t *A, int K, int kk, u64 *list) {
+    const int lane = threadIdx.x & 31;
+    const uint4 *A4 = reinterpret_cast<const uint4 *>(A);
+    const int nv = K >> 2, its = (nv + 31) >> 5;
+    uint32_t gm[kWParts];
+#pragma unroll
+    for (int q = 0; q < kWParts; ++q) {
+        uint32_t mx = 0u;
+        const int hi = its * (q + 1) / kWParts;
+#pragma unroll 4
+        for (int t = its * q / kWParts; t < hi; ++t) {
+            const int i = t * 32 + lane;
+            const uint4 v = i < nv ? __ldcg(A4 + i) : make_uint4(0u, 0u, 0u, 0u);
+            mx = max(mx, max(max(v.x, v.y), max(v.z, v.w)));
+        }
+        gm[q] = mx;
+    }
+    int groups = 0;
+#pragma unroll
+    for (int q = 0; q < kWParts; ++q) groups += gm[q] != 0u;
+    groups = (int)__reduce_add_sync(kFull, groups);
+    int cnt;
+    if (groups < kk) return -1;
+    const uint32_t tau = warp_kth<kWParts>(gm, groups, kk, &cnt);
+    int total = 0;
+    for (int t0 = 0; t0 < its; t0 += 32) {   // 4096 keys: four masks of 8 rounds
+        uint32_t hit[4];
+        int mine = 0;
+#pragma unroll
+        for (int w = 0; w < 4; ++w) {
+            uint32_t m = 0u;
+#pragma unroll
+            for (int u = 0; u < 8; ++u) {
+                const int i = (t0 + 8 * w + u) * 32 + lane;
+                if (i < nv) {
+                    const uint4 v = __ldcg(A4 + i);
+                    m |= (uint32_t)(v.x >= tau) << (4 * u) | (uint32_t)(v.y >= tau) << (4 * u + 1) |
+                         (uint32_t)(v.z >= tau) << (4 * u + 2) |
+                         (uint32_t)(v.w >= tau) << (4 * u + 3);
+                }
+            }
+            hit[w] = m;
+            mine += __popc(m);
+        }
+        const int incl = warp_scan(mine);
+        int at = total + incl - mine;
+        total += __shfl_sync(kFull, incl, 31);
+        if (total > kWCap) return -1;   // uniform
+#pragma unroll
+        for (int w = 0; w < 4; ++w)
+            for (uint32_t m = hit[w]; m; m &= m - 1u) {
+                const int bt = __ffs(m) - 1;
+                const int i = 4 * ((t0 + 8 * w + (bt >> 2)) * 32 + lane) + (bt & 3);
+                list[at++] = comp_of(A[i], (uint32_t)i);
+            }
+    }
+    return total;
+}
+
+// The k <= 64 positions of sel in increasing order.
+__device__ __forceinline__ void warp_sort_positions(int *sel, int k) {
+    const int lane = threadIdx.x & 31;
+    uint32_t x0 = 2 * lane < k ? (uint32_t)sel[2 * lane] : 0xffffffffu;
+    uint32_t x1 = 2 * lane + 1 < k ? (uint32_t)sel[2 * lane + 1] : 0xffffffffu;
+#pragma unroll
+    for (int blk = 2; blk <= 64; blk <<= 1)
+#pragma unroll
+        for (int st = blk >> 1; st > 0; st >>= 1) {
+            const bool up = ((2 * lane) & blk) == 0;   // ascending block
+            if (st == 1) {
+                const uint32_t a = min(x0, x1), b = max(x0, x1);
+                x0 = up ? a : b;
+                x1 = up ? b : a;
+            } else {
+                const uint32_t o0 = __shfl_xor_sync(kFull, x0, st >> 1);
+                const uint32_t o1 = __shfl_xor_sync(kFull, x1, st >> 1);
+                const bool lo = (((2 * lane) & st) == 0) == up;
+                x0 = lo ? min(x0, o0) : max(x0, o0);
+                x1 = lo ? min(x1, o1) : max(x1, o1);
+            }
+        }
+    __syncwarp();   // every position has been read
+    if (2 * lane < k) sel[2 * lane] = (int)x0;
+    if (2 * lane + 1 < k) sel[2 * lane + 1] = (int)x1;
+    __syncwarp();
+}
+
+// A warp's shared memory.  R: row pairs, [k / 2][RM][2] (row 2 t + e's entry
+// b at t 2 RM + 2 b + e); srow and scol [k][RM], S_row and S_col; entries past
+// the rank are 0.
+struct WarpSel {
+    u64 *list[2];   // [kWCap] each; the final candidates (kWTop) use both
+    u64 *top;       // [kWMaxK] the top m; before it, the final candidates' places
+    float *q;       // [2][D_k]
+    int *sel[2];    // [kWMaxK] survivors by increasing position
+    float *R, *srow, *scol;   // scol right behind srow
+};
+static_assert(kWTop <= 2 * kWCap, "the final candidates fit the axes' lists");
+
+constexpr int kWTopWords = kWMaxK > kWTop / 4 ? kWMaxK : kWTop / 4;   // of 8 bytes
+__host__ __device__ inline size_t warp_sel_bytes(const Dims &d, int rm) {
+    return 8 * (2 * kWCap + kWTopWords) + 4 * (2 * (size_t)d.d_k + 2 * kWMaxK) +
+           4 * (size_t)kWMaxK * rm * 3;
+}
+__device__ __forceinline__ WarpSel carve_warp(const Dims &d, int rm, unsigned char *base) {
+    WarpSel W;
+    W.list[0] = reinterpret_cast<u64 *>(base);
+    W.list[1] = W.list[0] + kWCap;
+    W.top = W.list[1] + kWCap;
+    W.R = reinterpret_cast<float *>(W.top + kWTopWords);
+    W.srow = W.R + kWMaxK * rm;
+    W.scol = W.srow + kWMaxK * rm;
+    W.q = W.scol + kWMaxK * rm;
+    W.sel[0] = reinterpret_cast<int *>(W.q + 2 * d.d_k);
+    W.sel[1] = W.sel[0] + kWMaxK;
+    return W;
+}
+
+// Lanes per survivor (2^lg), as in axis_survivors.
+__device__ __forceinline__ int survivor_lanes_log2(int k) {
+    int lg = 0;
+    while (lg < 5 && 2 * k * (2 << lg) <= kThreads) ++lg;
+    return lg;
+}
+
+// The row of survivor sv (rows 0 .. k - 1, then columns) in the key tables.
+__device__ __forceinline__ const uint4 *warp_row(const Dims &d, const Ptrs &p, int h, int sv,
+                                                 int *sel) {
+    const int s = sv >= d.k;
+    uint32_t pos = 0u;
+    if (sv < 2 * d.k) {
+        int *at = sel + (s ? kWMaxK + sv - d.k : sv);
+        pos = (uint32_t)*at;
+        if (pos >= (uint32_t)d.K) {   // never expected: record and skip
+            atomicOr(p.err, kErrInternal);
+            pos = 0u;
+            *at = 0;
+        }
+    }
+    const __nv_bfloat16 *keys = static_cast<const __nv_bfloat16 *>(s ? p.k_col : p.k_row);
+    return reinterpret_cast<const uint4 *>(keys + ((int64_t)h * d.K + pos) * d.d_k);
+}
+
+// R = S_row^T C of the row survivors, from the chunk scores (rows' in scol's
+// and srow's place beside it, see WarpSel); returns whether R and S_col are
+// finite.  Row pairs past the last one, up to a multiple of kWParts, repeat
+// it, and so does the missing second row of an odd k.
+template <int RM>
+__device__ __forceinline__ bool warp_fold_rows(const Dims &d, const float *core, const WarpSel &W) {
+    const int lane = threadIdx.x & 31, k = d.k, r = d.r;
+    const int np = (k + 1) >> 1, npad = (np + kWParts - 1) / kWParts * kWParts;
+    bool fin = true;
+    for (int i = lane; i < 2 * npad; i += 32) {
+        const int sv = min(i < 2 * np ? i : 2 * np - 2 + (i & 1), k - 1);
+        float S[RM];
+#pragma unroll
+        for (int a = 0; a < RM; ++a) {
+            S[a] = W.srow[sv * RM + a];
+            if (i < k) fin = fin && fabsf(W.scol[i * RM + a]) < INFINITY;
+        }
+#pragma unroll
+        for (int b = 0; b < RM; ++b) {
+            float v = 0.f;
+            if (b < r)
+#pragma unroll
+                for (int a = 0; a < RM; ++a)
+                    if (a < r) v = fmaf(S[a], core[a * r + b], v);
+            W.R[((i >> 1) * RM + b) * 2 + (i & 1)] = v;
+            fin = fin && fabsf(v) < INFINITY;
+        }
+    }
+    return __all_sync(kFull, fin);
+}
+
+// The query's place in W.q for the chunk scores below: vectors u and u + 1
+// (u even) of a lane interleaved, so that a 16-byte read gives two elements
+// of each.
+__device__ __forceinline__ int paired_q(int c, int lg) {
+    const int iv = c >> 3, u = iv >> lg, sub = iv & ((1 << lg) - 1);
+    return ((((u >> 1) << lg) + sub) << 4) + 2 * (c & 7) + (u & 1);
+}
+
+// The 2k survivors' chunk scores (bf16 rows of whole 16-byte vectors): G
+// lanes per survivor and the order of the sums as in axis_survivors.  A lane
+// takes NV vectors of its row, NV / CH of each of the CH chunks, two at a
+// time (packed fp32; the sums of the two stay apart), and asks for the next
+// survivor's vector as soon as it has used one, so that NV loads a lane stay
+// in flight.  The scores go to srow [2 kWMaxK][RM] (scol is its second
+// half), zeros past the rank.
+template <int RM, int NV, int CH>
+__device__ __forceinline__ void warp_survivors(const Dims &d, const Ptrs &p, int h, int lg,
+                                               const WarpSel &W) {
+    const int lane = threadIdx.x & 31, G = 1 << lg, sub = lane & (G - 1), per = 32 >> lg;
+    const int n = 2 * d.k;
+    int sv = lane >> lg;
+    const uint4 *row = warp_row(d, p, h, sv, W.sel[0]) + sub;
+    const uint64_t pol = key_row_policy();
+    uint4 buf[NV];
+#pragma unroll
+    for (int u = 0; u < NV; ++u) buf[u] = ld_key_row(row + (u << lg), pol);
+#pragma unroll 1
+    for (int s0 = 0; s0 < n; s0 += per, sv += per) {
+        const bool more = s0 + per < n;   // uniform
+        row = warp_row(d, p, h, sv + per, W.sel[0]) + sub;   // (its first row past the last)
+        const float *q = W.q + (sv >= d.k && sv < n ? d.d_k : 0) + (sub << 4);
+        float S[RM];
+#pragma unroll
+        for (int a = 0; a < RM; ++a) S[a] = 0.f;
+        // NC vector pairs at a time: their chains of sums interleave
+        constexpr int NC = NV >= 4 ? 2 : 1;
+#pragma unroll
+        for (int u0 = 0; u0 < NV; u0 += 2 * NC) {
+            u64 pv[NC];
+#pragma unroll
+            for (int c = 0; c < NC; ++c) pv[c] = 0ull;   // (0, 0)
+#pragma unroll
+            for (int w = 0; w < 4; ++w)   // elements 2 w and 2 w + 1 of the vectors
+#pragma unroll
+                for (int c = 0; c < NC; ++c) {
+                    const int u = u0 + 2 * c;
+                    const uint32_t x = (&buf[u].x)[w], y = (&buf[u + 1].x)[w];
+                    const ulonglong2 q2 = *reinterpret_cast<const ulonglong2 *>(
+                        q + ((u >> 1) << (lg + 4)) + 4 * w);
+                    pv[c] = fma2(pack2(__uint_as_float(x << 16), __uint_as_float(y << 16)), q2.x,
+                                 pv[c]);
+                    pv[c] = fma2(pack2(__uint_as_float(x & 0xffff0000u),
+                                       __uint_as_float(y & 0xffff0000u)),
+                                 q2.y, pv[c]);
+                }
+#pragma unroll
+            for (int u = u0; u < u0 + 2 * NC; ++u) ld_key_row_if(buf[u], row + (u << lg), pol, more);
+#pragma unroll
+            for (int c = 0; c < NC; ++c) {
+                const int u = u0 + 2 * c;
+                const float2 v = unpack2(pv[c]);
+                S[u * CH / NV] += v.x;
+                S[(u + 1) * CH / NV] += v.y;
+            }
+        }
+#pragma unroll
+        for (int a = 0; a < CH; ++a)
+            for (int off = G >> 1; off > 0; off >>= 1) S[a] += __shfl_xor_sync(kFull, S[a], off);
+        if (sub == 0 && sv < n) {
+            float *dst = W.srow + (sv < d.k ? sv : kWMaxK + sv - d.k) * RM;
+#pragma unroll
+            for (int a = 0; a < RM; ++a) dst[a] = S[a];
+        }
+    }
+}
+
+// The same for any number of vectors and chunks (the query in plain order).
+template <int RM>
+__device__ __noinline__ void warp_survivors_any(const Dims &d, const Ptrs &p, int h, int lg,
+                                                const WarpSel &W) {
+    const int lane = threadIdx.x & 31, G = 1 << lg, sub = lane & (G - 1), per = 32 >> lg;
+    const int n = 2 * d.k, nvec = d.d_k >> 3;
+    const float inv_dk = 1.f / (float)d.dk;   // see axis_survivors
+#pragma unroll 1
+    for (int s0 = 0; s0 < n; s0 += per) {
+        const int sv = s0 + (lane >> lg);
+        const uint4 *row = warp_row(d, p, h, sv, W.sel[0]);
+        const float *q = W.q + (sv >= d.k && sv < n ? d.d_k : 0);
+        float S[RM];
+#pragma unroll
+        for (int a = 0; a < RM; ++a) S[a] = 0.f;
+#pragma unroll 2
+        for (int iv = sub; iv < nvec; iv += G) {
+            float f[8];
+            unpack16<__nv_bfloat16>(ld_key_row(row + iv), f);
+            float pv = 0.f;
+#pragma unroll
+            for (int e = 0; e < 8; ++e) pv = fmaf(f[e], q[iv * 8 + e], pv);
+            const int al = (int)(((float)(iv * 8) + 0.5f) * inv_dk);
+#pragma unroll
+            for (int a = 0; a < RM; ++a) S[a] += a == al ? pv : 0.f;
+        }
+#pragma unroll
+        for (int a = 0; a < RM; ++a)
+            for (int off = G >> 1; off > 0; off >>= 1) S[a] += __shfl_xor_sync(kFull, S[a], off);
+        if (sub == 0 && sv < n) {
+            float *dst = W.srow + (sv < d.k ? sv : kWMaxK + sv - d.k) * RM;
+#pragma unroll
+            for (int a = 0; a < RM; ++a) dst[a] = S[a];
+        }
+    }
+}
+
+// RM >= r: 2 or 4 (PKM: 2).  Returns false when the (token, head) is left to
+// select_block.
+template <int RM, bool PKM, bool LISTS>
+__device__ __forceinline__ bool select_warp(const Dims &d, const Ptrs &p, int bh,
+                                            const WarpSel &W) {
+    const int lane = threadIdx.x & 31;
+    const int b = bh / d.H, h = bh - b * d.H;
+    const int k = d.k, m = d.m, K = d.K, D = d.d_k;
+    // the vectors a lane takes of a survivor's row, when they split evenly
+    // over the G lanes and the chunks (else 0)
+    constexpr int CH = PKM ? 1 : RM;
+    const int lg = survivor_lanes_log2(k);
+    int nv = D >> (3 + lg);
+    if (nv << (3 + lg) != D || d.r != CH || nv % CH || (nv & 1)) nv = 0;
+    const bool paired = nv == 8 || nv == 4 || (nv == 2 && CH <= 2);
+    // the row and column query of this (token, head)
+    const int HD = d.H * D;
+    for (int e = 4 * lane; e < 2 * D; e += 128) {
+        const int axis = e >= D, c = e - axis * D;
+        const int a = (axis == 1 && d.A == 2) ? 1 : 0;
+        const float4 v = *reinterpret_cast<const float4 *>(
+            p.q_part + ((int64_t)a * d.B + b) * HD + h * D + c);
+        if (paired) {
+            float *dst = W.q + axis * D + paired_q(c, lg);
+            dst[0] = v.x;
+            dst[2] = v.y;
+            dst[4] = v.z;
+            dst[6] = v.w;
+        } else {
+            *reinterpret_cast<float4 *>(W.q + e) = v;
+        }
+    }
+    // Eq. 8-9: the top k of each axis
+    int c[2];
+    const int64_t li = (int64_t)bh * 2;
+    if (LISTS) {
+        if (!warp_load_lists(p.gstat + li * d.n_segs, p.cand + li * d.n_segs * kSeg, d.n_segs,
+                             W.list[0], W.list[1], c))
+            return false;
+    } else {
+        for (int s = 0; s < 2; ++s)
+            c[s] = warp_scan_keys(p.akey + (li + s) * K, K, k, W.list[s]);
+    }
+    if (c[0] < k || c[1] < k) return false;   // uniform
+    __syncwarp();
+#pragma unroll 1
+    for (int s = 0; s < 2; ++s) {
+        int *sel = W.sel[0] + s * kWMaxK;
+        const u64 *list = W.list[0] + s * kWCap;
+        auto put = [&](int i, u64 x) { sel[i] = (int)pos_of(x); };
+        const int n = s ? c[1] : c[0];
+        if (n <= 96) warp_top<3>(list, n, k, put);
+        else warp_top<kWCap / 32>(list, n, k, put);
+        __syncwarp();
+        if (!LISTS) warp_sort_positions(sel, k);
+    }
+    // the survivors' chunk scores (Eq. 4)
+    const float *core = p.core + (int64_t)h * d.r * d.r;
+    if (paired && nv == 8) warp_survivors<RM, 8, CH>(d, p, h, lg, W);
+    else if (paired && nv == 4) warp_survivors<RM, 4, CH>(d, p, h, lg, W);
+    else if (paired) warp_survivors<RM, 2, (CH <= 2 ? CH : 1)>(d, p, h, lg, W);   // RM = 2
+    else warp_survivors_any<RM>(d, p, h, lg, W);
+    __syncwarp();
+    if (!warp_fold_rows<RM>(d, core, W)) return false;
+    __syncwarp();
+
+    // Eq. 10 on the k x k pairs, twice.  Lane l holds columns l and l + 32
+    // (a missing second column repeats the first, which changes no maximum).
+    const bool col0 = lane < k, col1 = lane + 32 < k;
+    const bool wide = k > 32;   // uniform
+    u64 sc[RM][2];
+#pragma unroll
+    for (int be = 0; be < RM; ++be) {
+        const float v0 = W.scol[(col0 ? lane : 0) * RM + be];
+        const float v1 = col1 ? W.scol[(lane + 32) * RM + be] : v0;
+        sc[be][0] = pack2(v0, v0);
+        sc[be][1] = pack2(v1, v1);
+    }
+    auto scores = [&](int t, u64 (&g)[2]) {   // rows 2 t, 2 t + 1 of both columns
+        u64 ra[RM];
+#pragma unroll
+        for (int be = 0; be < RM; be += 2) {
+            const ulonglong2 v = *reinterpret_cast<const ulonglong2 *>(W.R + (t * RM + be) * 2);
+            ra[be] = v.x;
+            ra[be + 1] = v.y;
+        }
+#pragma unroll
+        for (int cc = 0; cc < 2; ++cc) {
+            if (PKM) {
+                g[cc] = add2(ra[0], sc[0][cc]);
+            } else {
+                g[cc] = mul2(ra[0], sc[0][cc]);
+#pragma unroll
+                for (int be = 1; be < RM; ++be) g[cc] = fma2(ra[be], sc[be][cc], g[cc]);
+            }
+        }
+    };
+    // Part q of a lane is the row pairs [q tp, (q + 1) tp), tp <= 4 (past the
+    // last one, repeats of it: they count in the last real part only).
+    const int np = (k + 1) >> 1, tp = (np + kWParts - 1) / kWParts;
+    uint32_t gk[kWParts];
+    bool fin = true;
+    {
+        float gm[kWParts];
+#pragma unroll
+        for (int q = 0; q < kWParts; ++q) gm[q] = -INFINITY;
+#pragma unroll 1
+        for (int j = 0; j < tp; ++j) {
+#pragma unroll
+            for (int q = 0; q < kWParts; ++q) {
+                u64 g[2];
+                scores(q * tp + j, g);
+                const float2 x = unpack2(g[0]), y = unpack2(g[1]);
+                gm[q] = fmaxf(gm[q], fmaxf(x.x, x.y));
+                if (wide) gm[q] = fmaxf(gm[q], fmaxf(y.x, y.y));
+            }
+        }
+#pragma unroll
+        for (int q = 0; q < kWParts; ++q) {
+            const bool real = col0 && q * tp < np;
+            fin = fin && fabsf(gm[q]) < INFINITY;
+            gk[q] = real ? f2ord(gm[q]) : 0u;
+        }
+    }
+    if (!__all_sync(kFull, fin)) return false;   // an overflowed product
+    const int groups = min(k, 32) * ((np + tp - 1) / tp);
+    int cnt;
+    const bool all = groups < m;   // (small k) every pair is a candidate
+    const float tau = all ? 0.f : ord2f(warp_kth<kWParts>(gk, groups, m, &cnt, m >> 3));
+    // masks of the pairs >= tau: a score below it leaves a sign bit in
+    // g - tau (0 - tau turns a zero bound positive, so that -0 and +0 tie).
+    // Part q's mask holds tp row pairs of 4 pairs (rows 2 t, 2 t + 1 of
+    // column 0, then of column 1), the last one pushed in the low bits.
+    const u64 nt = pack2(0.f - tau, 0.f - tau);
+    uint32_t below[kWParts];
+#pragma unroll
+    for (int q = 0; q < kWParts; ++q) below[q] = 0u;
+#pragma unroll 1
+    for (int j = 0; j < tp; ++j) {
+#pragma unroll
+        for (int q = 0; q < kWParts; ++q) {
+            u64 g[2];
+            scores(q * tp + j, g);
+            const float2 x = unpack2(add2(g[0], nt)), y = unpack2(add2(g[1], nt));
+            uint32_t m4 = below[q];
+            m4 = __funnelshift_l(__float_as_uint(x.x), m4, 1);
+            m4 = __funnelshift_l(__float_as_uint(x.y), m4, 1);
+            m4 = __funnelshift_l(__float_as_uint(y.x), m4, 1);
+            below[q] = __funnelshift_l(__float_as_uint(y.y), m4, 1);
+        }
+    }
+    const int nb = 4 * tp;   // bits a part, <= 16
+    const uint32_t cols = !col0 ? 0u : col1 ? 0xffffu : 0xccccu;   // bits 4 x + 3, + 2: column 0
+    uint32_t hit[kWParts / 2];   // parts 2 w (high half) and 2 w + 1
+    int mine = 0;
+#pragma unroll
+    for (int w = 0; w < kWParts / 2; ++w) {
+        hit[w] = 0u;
+#pragma unroll
+        for (int z = 0; z < 2; ++z) {
+            const int q = 2 * w + z, miss = max(0, min(tp, (q + 1) * tp - np));   // repeats
+            uint32_t m4 = all ? 0xffffu : ~below[q];
+            m4 &= cols & ((1u << nb) - 1u) & ~((1u << 4 * miss) - 1u);
+            // the repeated row of an odd k: its pair's second row
+            if ((k & 1) && q * tp < np && (q + 1) * tp >= np) m4 &= ~(5u << 4 * miss);
+            hit[w] = hit[w] << 16 | m4;
+        }
+        mine += __popc(hit[w]);
+    }
+    const int incl = warp_scan(mine);
+    const int nc = __shfl_sync(kFull, incl, 31);
+    if (nc > kWTop || nc < m) return false;   // uniform
+    u64 *const list = W.list[0];
+    // the hits' places (lane and bit), packed, then a hit a lane: a hot column
+    // has many, and its lane would work them out alone
+    uint16_t *const code = reinterpret_cast<uint16_t *>(W.top);   // [kWTop]
+    int at = incl - mine;
+#pragma unroll
+    for (int w = 0; w < kWParts / 2; ++w)
+        for (uint32_t mk = hit[w]; mk; mk &= mk - 1u)
+            code[at++] = (uint16_t)(lane << 7 | w << 5 | (__ffs(mk) - 1));
+    __syncwarp();
+#pragma unroll 1
+    for (int i = lane; i < nc; i += 32) {
+        const int cd = code[i], bt = cd & 31;
+        // bit 4 x + 3 - e of a part: row pair tp - 1 - x, e = 2 column + row
+        const int q = 2 * (cd >> 5 & 3) + (bt < 16), x = bt & 15, e = 3 - (x & 3);
+        const int t = q * tp + tp - 1 - (x >> 2), z = e & 1, jj = (cd >> 7) + 32 * (e >> 1);
+        const float *Rt = W.R + t * 2 * RM + z, *Sj = W.scol + jj * RM;
+        float g = PKM ? Rt[0] + Sj[0] : Rt[0] * Sj[0];
+        if (!PKM) {
+#pragma unroll
+            for (int be = 1; be < RM; ++be) g = fmaf(Rt[2 * be], Sj[be], g);
+        }
+        list[i] = comp_of(f2ord(g), (uint32_t)((2 * t + z) * k + jj));
+    }
+    __syncwarp();
+    // the top m, sorted (lane l ends with ranks 2 l and 2 l + 1)
+    u64 *const top = W.top;
+    {
+        auto put = [&](int i, u64 x) { top[i] = x; };
+        if (nc <= 128) warp_top<4>(list, nc, m, put);
+        else if (nc <= 224) warp_top<7>(list, nc, m, put);
+        else warp_top<kWTop / 32>(list, nc, m, put);
+    }
+    __syncwarp();
+    u64 x0 = 2 * lane < m ? top[2 * lane] : 0ull, x1 = 2 * lane + 1 < m ? top[2 * lane + 1] : 0ull;
+#pragma unroll
+    for (int blk = 2; blk <= 64; blk <<= 1)
+#pragma unroll
+        for (int st = blk >> 1; st > 0; st >>= 1) {
+            const bool down = ((2 * lane) & blk) == 0;   // descending block
+            if (st == 1) {
+                const bool sw = (x0 < x1) == down;
+                const u64 a = sw ? x1 : x0, z = sw ? x0 : x1;
+                x0 = a;
+                x1 = z;
+            } else {
+                const u64 o0 = __shfl_xor_sync(kFull, x0, st >> 1);
+                const u64 o1 = __shfl_xor_sync(kFull, x1, st >> 1);
+                const bool big = (((2 * lane) & st) == 0) == down;
+                x0 = (x0 > o0) == big ? x0 : o0;
+                x1 = (x1 > o1) == big ? x1 : o1;
+            }
+        }
+
+    // weights (raw scores, or PKM's softmax), shuffle, outputs
+    float gmax = 0.f, z = 0.f;
+    if (d.act == ULTRAMEM_ACT_SOFTMAX) {
+        gmax = ord2f(key_of(__shfl_sync(kFull, x0, 0)));
+        __syncwarp();   // top has been read
+        if (2 * lane < m) top[2 * lane] = x0;
+        if (2 * lane + 1 < m) top[2 * lane + 1] = x1;
+        __syncwarp();
+        for (int e = lane; e < m; e += 32) z += __expf(ord2f(key_of(top[e])) - gmax);
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) z += __shfl_xor_sync(kFull, z, off);
+    }
+    const int64_t base = (int64_t)bh * m;
+    const uint32_t N = (uint32_t)d.N;
+    const uint32_t row_bytes = (uint32_t)d.d_v * 2u;
+    const bool prefetch = (uint64_t)d.B * d.H * m * row_bytes <= kPrefetchMaxBytes;
+    const float inv_k = 1.f / (float)k;   // c / k as in select_block's pairs
+    // a lane's two winners together: ranks e and e + 1
+    const int e = 2 * lane;
+    if (e >= m) return true;
+    const bool two = e + 1 < m;
+    int ii[2], jj[2], prow[2], pb[2];
+    int64_t v[2];
+    float w[2];
+#pragma unroll
+    for (int z2 = 0; z2 < 2; ++z2) {
+        const u64 x = z2 && two ? x1 : x0;
+        const int cc = (int)pos_of(x);
+        ii[z2] = (int)(((float)cc + 0.5f) * inv_k);
+        jj[z2] = cc - ii[z2] * k;
+        v[z2] = (int64_t)W.sel[0][ii[z2]] * K + W.sel[1][jj[z2]];
+        const float g = ord2f(key_of(x));
+        w[z2] = d.act == ULTRAMEM_ACT_SOFTMAX ? __expf(g - gmax) / z : g;
+        const uint32_t vs = (uint32_t)shuffle_address(d, p.perm, (uint64_t)v[z2]);   // Eq. 14
+        pb[z2] = (int)(vs / N);
+        prow[z2] = (int)(vs - (uint32_t)pb[z2] * N);
+    }
+    const int64_t at0 = base + e;
+    // 8-byte stores when every (token, head) starts on 8 bytes
+    const bool even = two && (m & 1) == 0;
+    auto put2 = [&](auto *dst, auto y0, auto y1, bool vec) {
+        using Y = decltype(y0);
+        struct alignas(2 * sizeof(Y)) Two {
+            Y a, b;
+        };
+        if (vec) {
+            *reinterpret_cast<Two *>(dst + at0) = Two{y0, y1};
+        } else {
+            dst[at0] = y0;
+            if (two) dst[at0 + 1] = y1;
+        }
+    };
+    put2(p.sel_row, prow[0], prow[1], even);
+    put2(p.sel_p, pb[0], pb[1], even);
+    if (p.idx_out)
+        put2(p.idx_out, v[0], v[1], even && ((uintptr_t)p.idx_out & 15) == 0);
+    if (d.nc == 1) {
+        put2(p.sel_w, w[0], w[1], even);
+        if (p.w_out) put2(p.w_out, w[0], w[1], even && ((uintptr_t)p.w_out & 7) == 0);
+    } else {
+        const int r = d.r;
+#pragma unroll
+        for (int z2 = 0; z2 < 2; ++z2) {
+            if (z2 && !two) break;
+            for (int ci = 0; ci < d.nc; ++ci) {   // Eq. 16-17, as in select_block
+                const float *Cc = p.cores + ((int64_t)h * d.nc + ci) * r * r;
+                float gi = 0.f;
+#pragma unroll
+                for (int a = 0; a < RM; ++a) {
+                    if (a < r) {
+                        float cs = 0.f;
+#pragma unroll
+                        for (int be = 0; be < RM; ++be)
+                            if (be < r) cs = fmaf(Cc[a * r + be], W.scol[jj[z2] * RM + be], cs);
+                        gi = fmaf(W.srow[ii[z2] * RM + a], cs, gi);
+                    }
+                }
+                p.sel_w[(at0 + z2) * d.nc + ci] = gi;
+                if (p.w_out) p.w_out[(at0 + z2) * d.nc + ci] = gi;
+            }
+        }
+    }
+    if (prefetch) {   // the gather reads these rows next
+        const unsigned char *V = static_cast<const unsigned char *>(p.values);
+        prefetch_l2(V + (size_t)prow[0] * row_bytes, row_bytes);
+        if (two) prefetch_l2(V + (size_t)prow[1] * row_bytes, row_bytes);
+    }
+    return true;
+}
+
+// A (token, head) that its warp left to the block.
+template <int RM>
+__device__ __noinline__ void select_left(const Dims &d, const Ptrs &p, int bh,
+                                         unsigned char *smem) {
+    SelShared &sh = *reinterpret_cast<SelShared *>(smem);
+    select_block<__nv_bfloat16, 4, (RM > 2 ? kMaxR : 2), false, false>(
+        d, p, bh, smem + sizeof(SelShared), sh);
+}
+
+template <int RM, bool PKM, bool LISTS>
+__global__ void __launch_bounds__(kThreads, 4) select_warp_kernel(Dims d, Ptrs p) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    __shared__ unsigned left;
+    const int warp = threadIdx.x >> 5;
+    const int bh = (int)blockIdx.x * kWarps + warp;
+    if (threadIdx.x == 0) left = 0u;
+    __syncthreads();
+    pdl_wait();
+    stamp_begin(p.stamp);
+    pdl_trigger();
+    if (bh < d.B * d.H) {   // warp-uniform
+        const WarpSel W = carve_warp(d, RM, smem_raw + warp * warp_sel_bytes(d, RM));
+        if (!select_warp<RM, PKM, LISTS>(d, p, bh, W) && (threadIdx.x & 31) == 0)
+            atomicOr(&left, 1u << warp);
+    }
+    __syncthreads();
+    for (unsigned t = left; t; t &= t - 1u) {   // uniform
+        select_left<RM>(d, p, (int)blockIdx.x * kWarps + __ffs(t) - 1, smem_raw);
+        __syncthreads();
+    }
     stamp_end(p.stamp);
 }
+
 
 // Candidate lists (Dims::cand), between the two scoring passes: the bound of
 // one (token, head, axis) per warp.  tau is the largest T whose low 16 bits
@@ -1293,7 +2143,7 @@ __global__ void __launch_bounds__(kThreads, MINB) select_kernel(Dims d, Ptrs p) 
 // lists by a few keys for twice the rounds.
 constexpr int kBoundWarps = 8;
 constexpr int kMaxGroupsPerLane = 32;   // G <= 1024 groups (K <= 16384 keys)
-static_assert(32 * kMaxGroupsPerLane == kMaxSegPerThread * kThreads, "one limit on G");
+static_assert(32 * kMaxGroupsPerLane == 4 * kMaxSegPerThread * kThreads, "one limit on K");
 template <int NQ>   // group maxima a lane holds, 32 NQ >= G
 __global__ void __launch_bounds__(32 * kBoundWarps) cand_bound_kernel(Dims d, Ptrs p) {
     pdl_wait();
@@ -1344,6 +2194,44 @@ __global__ void slots_kernel(Dims d, Ptrs p) {
 
 size_t select_smem_bytes(const Dims &d) { return sel_offsets(d).total; }
 
+// One warp per (token, head): bf16 rows of whole 16-byte vectors and chunks,
+// rank up to 4, k up to 64 and m <= k (the group maxima then bound the top m
+// well), the candidate lists or at least 1024 keys an axis, and enough
+// (token, head)s: a warp alone takes about 30 us for one whatever the grid
+// (35 with every key), the blocks longer grids.  Measured on GB300, a
+// retrieval, blocks -> warps: with the lists 64.5 -> 69.9 us at 800 (mid_4m,
+// 200 tokens), 62.4 -> 65.8 and 80.7 -> 77.4 at 1024 (K = 4096 and 5000),
+// 103.0 -> 100.4 at 1600; with every key (K = 2048) 42.4 -> 49.2 at 1000,
+// 82.0 -> 69.2 at 2000.
+constexpr int64_t kWarpGridLists = 1000, kWarpGridKeys = 1500;
+static bool warp_select_fits(const Dims &d, const Ptrs &p) {
+    return d.dtype == ULTRAMEM_BF16 && d.q_splits == 1 && d.r <= 4 && d.k <= kWMaxK &&
+           d.m <= d.k && d.d_k <= kWMaxD && d.dk % 8 == 0 &&
+           (((uintptr_t)p.k_row | (uintptr_t)p.k_col) & 15) == 0 &&
+           (d.cand || (d.K % 4 == 0 && d.K >= 1024)) &&
+           (int64_t)d.B * d.H > (d.cand ? kWarpGridLists : kWarpGridKeys);
+}
+template <int RM, bool PKM, bool LISTS>
+static cudaError_t launch_select_warp(Dims d, const Ptrs &p, cudaStream_t st) {
+    // what is left to the block reads its keys from L2 (16-byte loads)
+    if (!LISTS) d.stream_keys = 1;
+    const size_t block = sizeof(SelShared) + select_smem_bytes(d);
+    const size_t warps = kWarps * warp_sel_bytes(d, RM);
+    const int grid = (int)(((int64_t)d.B * d.H + kWarps - 1) / kWarps);
+    constexpr auto k = select_warp_kernel<RM, PKM, LISTS>;
+    // spread over the SMs (see spread_smem): the CTAs are placed while the
+    // scoring's hold most of them
+    const size_t sm =
+        spread_smem(block > warps ? block : warps, static_smem_of<k>(), grid);
+    return launch_kernel(d.pdl, k, grid, kThreads, sm, st, d, p);
+}
+template <bool LISTS>
+static cudaError_t launch_select_warps(const Dims &d, const Ptrs &p, cudaStream_t st) {
+    if (d.pkm) return launch_select_warp<2, true, LISTS>(d, p, st);
+    return d.r <= 2 ? launch_select_warp<2, false, LISTS>(d, p, st)
+                    : launch_select_warp<4, false, LISTS>(d, p, st);
+}
+
 template <typename T, int RM>
 static cudaError_t launch_select_t(const Dims &d, const Ptrs &p, size_t smem, cudaStream_t st) {
     if (d.B * d.H > 3 * 152 || d.cand)
@@ -1362,6 +2250,8 @@ static cudaError_t launch_select_t(const Dims &d, const Ptrs &p, size_t smem, cu
 }
 
 cudaError_t launch_select(const Dims &d, const Ptrs &p, cudaStream_t st) {
+    if (warp_select_fits(d, p))
+        return d.cand ? launch_select_warps<true>(d, p, st) : launch_select_warps<false>(d, p, st);
     const size_t smem = select_smem_bytes(d);
     if (d.dtype == ULTRAMEM_BF16)
         return d.r <= 2 ? launch_select_t<__nv_bfloat16, 2>(d, p, smem, st)
@@ -1412,12 +2302,23 @@ template <typename T, int RM> static cudaError_t allow_select() {
                                  (int)(kSmemPerCta - static_smem_of<select_kernel<T, 4, RM>>()));
     return e;
 }
+template <int RM, bool PKM, bool LISTS> static cudaError_t allow_select_warp() {
+    constexpr auto k = select_warp_kernel<RM, PKM, LISTS>;
+    return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                (int)(kSmemPerCta - static_smem_of<k>()));
+}
 
 cudaError_t configure_select(const Dims &) {
     cudaError_t e = allow_select<float, 2>();
     if (e == cudaSuccess) e = allow_select<float, kMaxR>();
     if (e == cudaSuccess) e = allow_select<__nv_bfloat16, 2>();
     if (e == cudaSuccess) e = allow_select<__nv_bfloat16, kMaxR>();
+    if (e == cudaSuccess) e = allow_select_warp<2, true, true>();
+    if (e == cudaSuccess) e = allow_select_warp<2, true, false>();
+    if (e == cudaSuccess) e = allow_select_warp<2, false, true>();
+    if (e == cudaSuccess) e = allow_select_warp<2, false, false>();
+    if (e == cudaSuccess) e = allow_select_warp<4, false, true>();
+    if (e == cudaSuccess) e = allow_select_warp<4, false, false>();
     return e;
 }
 

@@ -137,7 +137,9 @@ __device__ __forceinline__ void group_epilogue(const Op &op, const Tile &t, int 
             float v[16];
 #pragma unroll
             for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[half * 16 + i]);
-            g[cc * 2 + half] = op.group(t, row, cb + cc * 32 + half * 16, v, pre);
+            const int gi = cc * 2 + half;
+            g[gi] = op.group(t, row, cb + cc * 32 + half * 16, v, pre,
+                             gi % 4 ? g[gi > 0 ? gi - 1 : 0] : 0u);
         }
     }
     op.template store_groups<NG>(t, row, cb, g);
@@ -780,16 +782,17 @@ struct ScoreOp {
 // largest of those group maxima: k distinct groups hold a key >= tau, so
 // every key of the axis' top k is >= tau.  The second pass (kListCandidates)
 // recomputes the same keys (the same tiles, MMAs and order, so bit for bit)
-// and writes each key >= tau, as a (key, position) composite, into its
-// group's 16-entry segment of the (token, head, axis) list, and the group's
-// count over its maximum.  About 2 % of the keys land in the lists, and the
+// and writes each key >= tau, as a (key, position) composite, into the
+// (token, head, axis) list's segment of its 64 keys (which one thread owns),
+// and the segment's count.  About 2 % of the keys land in the lists, and the
 // selection gets 17-25 % shorter.  Measured on GB300 (step times, graph
 // replays): with 16 epilogue warps and 256-key tiles the two passes and
 // the bound cost less than that saves once each SM has about 3.5 of their
 // tiles (prefill of 16384 tokens 3255 -> 3083 us a step), more below (mid_4m
 // with 128 tokens 65.7 -> 80.4 us), so the layer picks the form by grid.
 enum { kListGroupMax = 1, kListCandidates = 2 };
-constexpr int kListGroup = 16;   // keys of a group; entries of a list segment
+constexpr int kListGroup = 16;   // keys of a group
+constexpr int kListSeg = 64;     // keys and entries of a list segment
 
 template <int Mode>
 struct ScoreListOp {
@@ -801,9 +804,10 @@ struct ScoreListOp {
     unsigned long long *stamp;   // profiling stamps of the stage, or null
     int B, H, K, kb_total;
     int G;                        // groups of 16 keys an axis
-    uint32_t *gstat;              // [B][H][2][G] group maxima, then group counts
+    int segs;                     // segments of 64 keys an axis
+    uint32_t *gstat;              // [B][H][2][G] group maxima; [B][H][2][segs] counts
     const uint32_t *tau;          // [B][H][2]
-    unsigned long long *cand;     // [B][H][2][G][16] composites
+    unsigned long long *cand;     // [B][H][2][segs][64] composites
     __device__ int cluster_splits() const { return 1; }
     int cluster_splits_host() const { return 1; }
     __device__ void store_sums(const Tile &, int, int, const float (&)[4]) const {}
@@ -828,13 +832,14 @@ struct ScoreListOp {
     }
     static constexpr bool kGroupEpilogue = true;
     // row: the token (TMEM lane); c: the tile column of the group's first
-    // key.  Returns the group's largest key (group maxima), or its count
-    // after writing its keys >= t to its segment (candidates).
-    __device__ uint32_t group(const Tile &tl, int row, int c, const float (&v)[16],
-                              uint32_t t) const {
+    // key.  Returns the group's largest key (group maxima), or, after writing
+    // its keys >= t (candidates), how many its segment holds so far, `had`
+    // of them from the segment's earlier groups.
+    __device__ uint32_t group(const Tile &tl, int row, int c, const float (&v)[16], uint32_t t,
+                              uint32_t had) const {
         const int n = tl.n0 + row;
         const int i0 = tl.m0 + c;
-        if (n >= B || i0 >= K) return 0u;
+        if (n >= B || i0 >= K) return Mode == kListCandidates ? had : 0u;
         const int valid = min(kListGroup, K - i0);
         // f2ord is monotone (-0 and +0 share a key), so the maximum and the
         // comparisons are taken on the fp32 scores and only kept keys are
@@ -848,22 +853,30 @@ struct ScoreListOp {
         } else {
             const float tf = ord2f(t);   // v >= tf  <=>  f2ord(v) >= t
             unsigned long long *seg =
-                cand + (((int64_t)n * H * 2 + tl.z) * G + i0 / kListGroup) * kListGroup;
-            uint32_t cnt = 0u;
+                cand + (((int64_t)n * H * 2 + tl.z) * segs + i0 / kListSeg) * kListSeg;
+            uint32_t cnt = had;
 #pragma unroll
             for (int j = 0; j < kListGroup; ++j)
                 if (j < valid && v[j] >= tf) seg[cnt++] = comp_of(f2ord(v[j]), (uint32_t)(i0 + j));
             return cnt;
         }
     }
-    // the NG groups from tile column c (a multiple of 16 NG): 16-byte stores
-    // when every row of gstat starts on 16 bytes (G a multiple of 4), else
-    // one store per group
+    // the NG groups from tile column c (a multiple of 16 NG).  Maxima: 16-byte
+    // stores when every row of gstat starts on 16 bytes (G a multiple of 4),
+    // else one store per group.  Candidates: the count of each segment (four
+    // groups).
     template <int NG>
     __device__ void store_groups(const Tile &tl, int row, int c, const uint32_t (&g)[NG]) const {
         const int n = tl.n0 + row;
         const int gi = (tl.m0 + c) / kListGroup;
         if (n >= B || gi >= G) return;
+        if constexpr (Mode == kListCandidates) {
+            uint32_t *cnt = gstat + ((int64_t)n * H * 2 + tl.z) * segs + gi / 4;
+#pragma unroll
+            for (int q = 0; q < NG / 4; ++q)
+                if (gi + 4 * q < G) cnt[q] = g[4 * q + 3];
+            return;
+        }
         uint32_t *dst = gstat + ((int64_t)n * H * 2 + tl.z) * G + gi;
         if ((G & 3) == 0) {
 #pragma unroll
@@ -1270,6 +1283,7 @@ static cudaError_t score_list_pass(const Dims &d, const Ptrs &p, const TcMaps &m
     op.K = d.K;
     op.kb_total = (d.d_k + kBlockK - 1) / kBlockK;
     op.G = d.n_groups;
+    op.segs = d.n_segs;
     op.gstat = p.gstat;
     op.tau = p.tau;
     op.cand = p.cand;
