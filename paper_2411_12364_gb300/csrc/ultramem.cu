@@ -448,12 +448,22 @@ ultramem_status run_cuda_core(ultramem_layer *L, const Dims &d0, Ptrs p, cudaStr
     {
         Ptrs pq = p0;
         if (d.conv_k > 0) pq.x = p.xs;   // the fp32 convolved rows
-        if ((e = um::launch_query(d, pq, d.conv_k > 0, st)) != cudaSuccess) return from_cuda(e);
+        Dims dq = d;
+        dq.pdl = d.conv_k > 0;   // a dependent of the convolution
+        if ((e = um::launch_query(dq, pq, d.conv_k > 0, !d.query_ln, st)) != cudaSuccess)
+            return from_cuda(e);
     }
-    if (d.query_ln) {
-        if ((e = um::launch_query_ln(d, p0, nullptr, 0, st)) != cudaSuccess) return from_cuda(e);
-        d.q_splits = 1;   // the normalised query is split 0
-    }
+    // every kernel after the first is a programmatic dependent launch of its
+    // predecessor; they all wait for it before they read or write
+    d.pdl = 1;
+    if (d.query_ln && (e = um::launch_query_ln(d, p0, nullptr, 0, st)) != cudaSuccess)
+        return from_cuda(e);
+    // the query is in split 0; the selection of fp32 storage takes the one
+    // summed in fp64
+    Ptrs ps = p;
+    if (d.dtype == ULTRAMEM_F32 && !d.query_ln && d.q_splits > 1)
+        ps.q_part += (size_t)d.A * d.B * d.H * d.d_k;
+    d.q_splits = 1;
     if (mode == kExact) {
         int n = 0;
         if ((e = um::launch_exact(d, p, p.idx_out, p.w_out, &n, st)) != cudaSuccess)
@@ -462,7 +472,7 @@ ultramem_status run_cuda_core(ultramem_layer *L, const Dims &d0, Ptrs p, cudaStr
         return ULTRAMEM_OK;
     }
     if ((e = um::launch_score(d, stage_ptrs(L, p, 1), st)) != cudaSuccess) return from_cuda(e);
-    if ((e = um::launch_select(d, stage_ptrs(L, p, 2), st)) != cudaSuccess) return from_cuda(e);
+    if ((e = um::launch_select(d, stage_ptrs(L, ps, 2), st)) != cudaSuccess) return from_cuda(e);
     *launches = 3 + extras;
     if (mode == kRetrieve) return ULTRAMEM_OK;
     if ((e = um::launch_gather(d, stage_ptrs(L, p, 3), st)) != cudaSuccess) return from_cuda(e);
@@ -856,6 +866,7 @@ ultramem_status ultramem_create(const ultramem_config *cfg, const ultramem_weigh
     if (e == cudaSuccess && L->exact_ok) e = um::configure_exact(d);
     if (e == cudaSuccess) e = um::configure_select(d);
     if (e == cudaSuccess) e = um::configure_gather(d);
+    if (e == cudaSuccess) e = um::configure_cuda_core();
     if (e != cudaSuccess) {
         free_workspace(ws);
         delete L;

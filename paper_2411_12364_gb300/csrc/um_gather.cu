@@ -15,15 +15,16 @@
 // Wider rows or more slots take the per-lane multi-block kernels below.  Row
 // loads bypass L1 (read-only path).
 //
-// fp32 storage accumulates in fp64 (products of two fp32 values are exact
-// there): the fp32 mode's outputs carry the working precision element by
-// element (see Dot2 in um_internal.cuh), and its projection reads fp32
-// pooled rows that are rounded once.
+// fp32 storage accumulates with compensated sums (Dot2; the general kernels in
+// fp64): the fp32 mode's outputs carry the working precision element by
+// element (see Dot2 in um_internal.cuh), and its projection reads fp32 pooled
+// rows that are rounded once.
 //
 // Multi-Core Scoring (Eq. 17): a slot has nc weights and weight i scales
 // columns [i*D_v/nc, (i+1)*D_v/nc) of the row.  Slices are whole 16-byte
 // vectors (D_v/nc is a multiple of 8), so a lane's vector lies in one slice
 // and the lane picks that slice's weight.
+#include "um_dot.cuh"
 #include "um_internal.cuh"
 
 namespace um {
@@ -191,18 +192,23 @@ size_t bucket_smem_bytes(const Dims &d, int warps) {
 // instead of the selection's sel_row / sel_p / sel_w, and each thread works
 // its slot out itself: the slots kernel before the gather, its launch and
 // the round trip of 12 bytes a slot through memory go.
-template <typename T, int THREADS, bool ADDR>
-__global__ void __launch_bounds__(THREADS, 1024 / THREADS) gather_bucket_kernel(Dims d, Ptrs p) {
-    constexpr int kBThreads = THREADS, kBWarps = THREADS / 32;
+// VPL: 16-byte vectors of a row that a lane owns (2: fp32 rows of up to 256
+// values; half as many rows in flight).  fp32 rows' fp64 sums take twice the
+// registers, so half as many CTAs per SM.
+template <typename T, int THREADS, bool ADDR, int VPL = 1>
+__global__ void __launch_bounds__(THREADS, (sizeof(T) == 4 ? 512 : 1024) / THREADS)
+    gather_bucket_kernel(Dims d, Ptrs p) {
+    constexpr int kBThreads = THREADS, kBWarps = THREADS / 32, kRows = kUnroll / VPL;
     extern __shared__ __align__(16) unsigned char gsm[];
     __shared__ int wcnt[kBWarps][kBMaxE];   // per warp and block: count, then offset
     __shared__ int tot[kBMaxE], start[kBMaxE];
     constexpr int EPV = 16 / sizeof(T);
-    using A = AccOf<T>;
     const int b = blockIdx.x, E = d.E, hm = d.H * d.m, Dv = d.d_v;
     const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
     const int64_t base = (int64_t)b * hm;
-    A *red = reinterpret_cast<A *>(gsm);                         // [kBWarps][D_v]
+    // the warps' sums [kBWarps][D_v]: fp32, or (fp32 storage) s and c of Dot2
+    using R = typename std::conditional<std::is_same<T, float>::value, float2, float>::type;
+    R *red = reinterpret_cast<R *>(gsm);
     int *row_s = reinterpret_cast<int *>(red + kBWarps * Dv);    // [hm] bucketed rows
     float *w_s = reinterpret_cast<float *>(row_s + hm);          // [hm][nc] their weights
     const int nc = d.nc;
@@ -266,45 +272,92 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS) gather_bucket_kernel(
     // warps [q*wpb, (q+1)*wpb) serve block q, each a contiguous share
     const int wpb = kBWarps / E;
     const int q = warp / wpb, sub = warp - q * wpb;
-    const bool active = lane * EPV < Dv;
-    const int wsel = nc == 1 || !active ? 0 : (lane * EPV) / (Dv / nc);   // this lane's slice
-    const T *V = static_cast<const T *>(p.values) + lane * EPV;
-    A acc[EPV];
+    bool active[VPL];
+    int wsel[VPL];   // the slice that a vector lies in
 #pragma unroll
-    for (int c = 0; c < EPV; ++c) acc[c] = 0;
+    for (int x = 0; x < VPL; ++x) {
+        const int c0 = (lane + 32 * x) * EPV;
+        active[x] = c0 < Dv;
+        wsel[x] = nc == 1 || !active[x] ? 0 : c0 / (Dv / nc);
+    }
+    const T *V = static_cast<const T *>(p.values) + lane * EPV;
+    constexpr bool kExact = std::is_same<T, float>::value;
+    float acc[kExact ? 1 : VPL][EPV];
+    dot::Dot2x2 ex[kExact ? VPL : 1][kExact ? EPV / 2 : 1];   // fp32 storage: pairs of columns
+    if constexpr (!kExact)
+#pragma unroll
+        for (int x = 0; x < VPL; ++x)
+#pragma unroll
+            for (int c = 0; c < EPV; ++c) acc[x][c] = 0.f;
     if (q < E) {
         const int n = tot[q], per = (n + wpb - 1) / wpb;
         const int lo = start[q] + min(n, sub * per), hi = start[q] + min(n, (sub + 1) * per);
-        for (int j0 = lo; j0 < hi; j0 += kUnroll) {
-            uint4 val[kUnroll];
-            float wu[kUnroll];
+        for (int j0 = lo; j0 < hi; j0 += kRows) {
+            uint4 val[kRows][VPL];
+            float wu[kRows][VPL];
 #pragma unroll
-            for (int u = 0; u < kUnroll; ++u) {
+            for (int u = 0; u < kRows; ++u) {
                 const int j = j0 + u;
                 const bool ok = j < hi;
-                wu[u] = ok ? w_s[j * nc + wsel] : 0.f;
-                val[u] = (ok && active) ? ld_stream(V + (int64_t)row_s[j] * Dv)
-                                        : make_uint4(0, 0, 0, 0);
+#pragma unroll
+                for (int x = 0; x < VPL; ++x) {
+                    wu[u][x] = ok ? w_s[j * nc + wsel[x]] : 0.f;
+                    val[u][x] = (ok && active[x])
+                                    ? ld_stream(V + (int64_t)row_s[j] * Dv + 32 * x * EPV)
+                                    : make_uint4(0, 0, 0, 0);
+                }
             }
 #pragma unroll
-            for (int u = 0; u < kUnroll; ++u) {
-                float f[EPV];
-                unpack<T>(val[u], f);
+            for (int u = 0; u < kRows; ++u)
 #pragma unroll
-                for (int c = 0; c < EPV; ++c) acc[c] = mul_add(wu[u], f[c], acc[c]);
-            }
+                for (int x = 0; x < VPL; ++x) {
+                    float f[EPV];
+                    unpack<T>(val[u][x], f);
+                    if constexpr (kExact) {
+                        const f2 w2 = pack2(wu[u][x], wu[u][x]), n2 = pack2(-wu[u][x], -wu[u][x]);
+#pragma unroll
+                        for (int c = 0; c < EPV; c += 2) ex[x][c / 2].add(w2, n2, pack2(f[c], f[c + 1]));
+                    } else {
+#pragma unroll
+                        for (int c = 0; c < EPV; ++c)
+                            acc[x][c] = mul_add(wu[u][x], f[c], acc[x][c]);
+                    }
+                }
         }
-        if (active)
 #pragma unroll
-            for (int c = 0; c < EPV; ++c) red[warp * Dv + lane * EPV + c] = acc[c];
+        for (int x = 0; x < VPL; ++x)
+            if (active[x])
+#pragma unroll
+                for (int c = 0; c < EPV; ++c) {
+                    R &dst = red[warp * Dv + (lane + 32 * x) * EPV + c];
+                    if constexpr (kExact) {
+                        const float2 sv = unpack2(ex[x][c / 2].s), cv = unpack2(ex[x][c / 2].c);
+                        dst = c & 1 ? make_float2(sv.y, cv.y) : make_float2(sv.x, cv.x);
+                    } else {
+                        dst = acc[x][c];
+                    }
+                }
     }
     __syncthreads();
     const int EDv = E * Dv;
     for (int i = t; i < EDv; i += kBThreads) {
         const int qq = i / Dv, c = i - qq * Dv;
-        A sum = 0;
-        for (int sb = 0; sb < wpb; ++sb) sum += red[(qq * wpb + sb) * Dv + c];
-        store_pooled<T>(d, p, b, i, (float)sum);
+        float sum;
+        if constexpr (kExact) {
+            Dot2 all;
+            for (int sb = 0; sb < wpb; ++sb) {
+                const float2 v = red[(qq * wpb + sb) * Dv + c];
+                Dot2 o;
+                o.s = v.x;
+                o.c = v.y;
+                all.merge(o);
+            }
+            sum = all.value_any();
+        } else {
+            sum = 0.f;
+            for (int sb = 0; sb < wpb; ++sb) sum += red[(qq * wpb + sb) * Dv + c];
+        }
+        store_pooled<T>(d, p, b, i, sum);
     }
     stamp_end(p.stamp);
 }
@@ -369,75 +422,65 @@ __global__ void __launch_bounds__(kThreads) gather_kernel(Dims d, Ptrs p) {
 }
 
 // proj_part[split][b][o] = sum over this split's slice of E*D_v of acc[b][c] W[c][o]
-// (W = the E projectors stacked: [E*D_v][D'_v]).  Tile 32 tokens x 64 outputs.
-template <typename T>
-__global__ void __launch_bounds__(kThreads) proj_kernel(Dims d, Ptrs p) {
-    const int Kd = d.E * d.d_v;
-    const int split = blockIdx.z;
+// (W = the E projectors stacked: [E*D_v][D'_v]); fp32 storage: compensated
+// sums (Dot2), each partial to the working precision.
+template <typename T, int TPT, int NP>
+__global__ void __launch_bounds__(dot::kThreads) proj_kernel(Dims d, Ptrs p) {
+    using Acc = dot::AccFor<T>;
+    using S = dot::Shape<TPT, NP>;
+    __shared__ dot::Stage<Acc, TPT, NP> st;
+    const int Kd = d.E * d.d_v, split = blockIdx.z;
     const int chunk = (Kd + d.p_splits - 1) / d.p_splits;
-    const int kb = split * chunk, ke = min(Kd, kb + chunk);
-    const int o0 = blockIdx.x * 64, b0 = blockIdx.y * 32;
-    const T *W = static_cast<const T *>(p.w_proj);
+    const int o0 = blockIdx.x * S::TN, b0 = blockIdx.y * S::TM;
+    pdl_wait();
     stamp_begin(p.stamp);
-    __shared__ float as[32][33];   // [c][token]
-    __shared__ float ws[32][65];   // [c][output]
-    const int tid = threadIdx.x, tx = tid % 16, ty = tid / 16;
-    // fp32 storage: compensated sums (Dot2), each partial to the working precision
-    constexpr bool kExact = std::is_same<T, float>::value;
-    float acc[2][4] = {};
-    Dot2 ex[kExact ? 2 : 1][kExact ? 4 : 1];
-    for (int k0 = kb; k0 < ke; k0 += 32) {
-        for (int e = tid; e < 32 * 32; e += kThreads) {
-            int bb = e / 32, kk = e % 32, b = b0 + bb, c = k0 + kk;
-            as[kk][bb] = (b < d.B && c < ke) ? p.acc[(int64_t)b * Kd + c] : 0.f;
-        }
-        for (int e = tid; e < 32 * 64; e += kThreads) {
-            int kk = e / 64, oo = e % 64, c = k0 + kk, o = o0 + oo;
-            ws[kk][oo] = (c < ke && o < d.d_out) ? to_f(W[(int64_t)c * d.d_out + o]) : 0.f;
-        }
-        __syncthreads();
-#pragma unroll 8
-        for (int kk = 0; kk < 32; ++kk) {
-            float a0 = as[kk][ty * 2], a1 = as[kk][ty * 2 + 1];
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                float wv = ws[kk][tx * 4 + j];
-                if constexpr (kExact) {
-                    ex[0][j].add(a0, wv);
-                    ex[1][j].add(a1, wv);
-                } else {
-                    acc[0][j] = fmaf(a0, wv, acc[0][j]);
-                    acc[1][j] = fmaf(a1, wv, acc[1][j]);
-                }
-            }
-        }
-        __syncthreads();
-    }
-    for (int i = 0; i < 2; ++i)
-        for (int j = 0; j < 4; ++j) {
-            int b = b0 + ty * 2 + i, o = o0 + tx * 4 + j;
-            float v = acc[i][j];
-            if constexpr (kExact) v = ex[i][j].value();
-            if (b < d.B && o < d.d_out)
-                p.proj_part[((int64_t)split * d.B + b) * d.d_out + o] = v;
-        }
+    pdl_trigger();
+    dot::Operands<float, T> o;
+    o.A = p.acc;
+    o.B = static_cast<const T *>(p.w_proj);
+    o.lda = Kd;
+    o.ldb = d.d_out;
+    o.M = d.B;
+    o.N = d.d_out;
+    o.kb = min(Kd, split * chunk);
+    o.ke = min(Kd, o.kb + chunk);
+    o.veca = ((Kd | chunk) & 3) == 0;   // acc is the library's, 16-byte aligned
+    o.vecb = (d.d_out & 3) == 0 && ((uintptr_t)o.B & (4 * sizeof(T) - 1)) == 0;
+    Acc acc[TPT][NP];
+    dot::tile<Acc, TPT, NP, false>(o, b0, o0, st, acc, [](int) {});
+    dot::each<Acc, TPT, NP>(acc, [&](int i, int j, float v) {
+        if (b0 + i < d.B && o0 + j < d.d_out)
+            p.proj_part[((int64_t)split * d.B + b0 + i) * d.d_out + o0 + j] = v;
+    });
     stamp_end(p.stamp);
 }
 
-// out = the sum of the split-K partials (in fp64 with fp32 storage: one
+// out = the sum of the split-K partials (fp32 storage: compensated, one
 // rounding of the output)
 template <typename T>
 __global__ void proj_reduce_kernel(Dims d, Ptrs p) {
     pdl_wait();
     stamp_begin(p.stamp);
     pdl_trigger();
-    using A = AccOf<T>;
     const int64_t total = (int64_t)d.B * d.d_out;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < total;
          i += (int64_t)gridDim.x * blockDim.x) {
-        A s = 0;
-        for (int sp = 0; sp < d.p_splits; ++sp) s += (A)p.proj_part[(int64_t)sp * total + i];
-        static_cast<T *>(p.out)[i] = from_f<T>((float)s);
+        float v[8], out;
+#pragma unroll
+        for (int sp = 0; sp < 8; ++sp)
+            v[sp] = sp < d.p_splits ? p.proj_part[(int64_t)sp * total + i] : 0.f;
+        if constexpr (std::is_same<T, float>::value) {
+            Dot2 sum;
+#pragma unroll
+            for (int sp = 0; sp < 8; ++sp) sum.two_sum_into(v[sp]);
+            out = sum.value_any();
+        } else {
+            out = 0.f;
+#pragma unroll
+            for (int sp = 0; sp < 8; ++sp)
+                if (sp < d.p_splits) out += v[sp];
+        }
+        static_cast<T *>(p.out)[i] = from_f<T>(out);
     }
     stamp_end(p.stamp);
 }
@@ -471,32 +514,46 @@ cudaError_t configure_gather(const Dims &) {
     if (e == cudaSuccess) e = allow_padded<gather_bucket_kernel<__nv_bfloat16, 512, false>>();
     if (e == cudaSuccess) e = allow_padded<gather_bucket_kernel<float, 256, false>>();
     if (e == cudaSuccess) e = allow_padded<gather_bucket_kernel<__nv_bfloat16, 256, false>>();
+    if (e == cudaSuccess) e = allow_padded<gather_bucket_kernel<float, 512, false, 2>>();
+    if (e == cudaSuccess) e = allow_padded<gather_bucket_kernel<float, 256, false, 2>>();
+    if (e == cudaSuccess) e = allow_padded<proj_kernel<float, 2, 2>>();
+    if (e == cudaSuccess) e = allow_padded<proj_kernel<float, 1, 1>>();
+    if (e == cudaSuccess) e = allow_padded<proj_kernel<__nv_bfloat16, 2, 2>>();
+    if (e == cudaSuccess) e = allow_padded<proj_kernel<__nv_bfloat16, 1, 1>>();
     if (e == cudaSuccess) e = allow_padded<gather_bucket_kernel<__nv_bfloat16, 512, true>>();
     if (e == cudaSuccess) e = allow_padded<gather_bucket_kernel<__nv_bfloat16, 256, true>>();
     return e;
 }
 
-// The bucketed gather, where it serves the layer's shape (*taken).
+// The bucketed gather, where it serves the layer's shape (*taken).  fp32 rows
+// of 33 to 64 vectors (D_v to 256) take two vectors a lane.
+template <typename T, bool ADDR, int VPL>
+static cudaError_t launch_bucket_v(const Dims &d, const Ptrs &p, bool *taken, cudaStream_t st) {
+    *taken = true;
+    // spread over the SMs (see spread_smem)
+    if (d.B <= 2 * 152 && d.H * d.m <= 512) {
+        constexpr auto k = gather_bucket_kernel<T, 512, ADDR, VPL>;
+        return launch_kernel(d.pdl, k, d.B, 512,
+                             spread_smem(bucket_smem_bytes(d, 16), static_smem_of<k>(), d.B), st,
+                             d, p);
+    }
+    if (d.H * d.m <= 256 && d.E <= 8) {
+        constexpr auto k = gather_bucket_kernel<T, 256, ADDR, VPL>;
+        return launch_kernel(d.pdl, k, d.B, 256,
+                             spread_smem(bucket_smem_bytes(d, 8), static_smem_of<k>(), d.B), st,
+                             d, p);
+    }
+    *taken = false;
+    return cudaSuccess;
+}
 template <typename T, bool ADDR>
 static cudaError_t launch_bucket(const Dims &d, const Ptrs &p, bool *taken, cudaStream_t st) {
     constexpr int epv = 16 / (int)sizeof(T);
-    *taken = true;
-    if (d.d_v / epv <= 32 && d.d_v % epv == 0 && d.E <= kBMaxE) {
-        // spread over the SMs (see spread_smem)
-        if (d.B <= 2 * 152 && d.H * d.m <= 512) {
-            constexpr auto k = gather_bucket_kernel<T, 512, ADDR>;
-            return launch_kernel(d.pdl, k, d.B, 512,
-                                 spread_smem(bucket_smem_bytes(d, 16), static_smem_of<k>(), d.B),
-                                 st, d, p);
-        }
-        if (d.H * d.m <= 256 && d.E <= 8) {
-            constexpr auto k = gather_bucket_kernel<T, 256, ADDR>;
-            return launch_kernel(d.pdl, k, d.B, 256,
-                                 spread_smem(bucket_smem_bytes(d, 8), static_smem_of<k>(), d.B),
-                                 st, d, p);
-        }
-    }
     *taken = false;
+    if (d.d_v % epv || d.E > kBMaxE) return cudaSuccess;
+    if (d.d_v / epv <= 32) return launch_bucket_v<T, ADDR, 1>(d, p, taken, st);
+    if constexpr (std::is_same<T, float>::value)
+        if (d.d_v / epv <= 64) return launch_bucket_v<T, ADDR, 2>(d, p, taken, st);
     return cudaSuccess;
 }
 
@@ -536,19 +593,28 @@ cudaError_t launch_gather(const Dims &d, const Ptrs &p, cudaStream_t st) {
     return launch_gather_t<float>(d, p, st);
 }
 
+template <typename T, int TPT, int NP>
+static cudaError_t launch_proj_t(const Dims &d, const Ptrs &p, cudaStream_t st) {
+    using S = dot::Shape<TPT, NP>;
+    dim3 grid((d.d_out + S::TN - 1) / S::TN, (d.B + S::TM - 1) / S::TM, d.p_splits);
+    // a dependent launch is spread over the SMs (see spread_smem)
+    constexpr auto k = proj_kernel<T, TPT, NP>;
+    const size_t sm = d.pdl ? spread_smem(0, static_smem_of<k>(), ctas_of(grid)) : 0;
+    cudaError_t e = launch_kernel(d.pdl, k, grid, dot::kThreads, sm, st, d, p);
+    if (e != cudaSuccess) return e;
+    const int64_t total = (int64_t)d.B * d.d_out;
+    const int64_t blocks = (total + 255) / 256;
+    return launch_kernel(d.pdl, proj_reduce_kernel<T>, (unsigned)(blocks < 4096 ? blocks : 4096),
+                         256, 0, st, d, p);
+}
+
 cudaError_t launch_proj(const Dims &d, const Ptrs &p, cudaStream_t st) {
-    dim3 grid((d.d_out + 63) / 64, (d.B + 31) / 32, d.p_splits);
-    int64_t total = (int64_t)d.B * d.d_out;
-    int rblocks = (int)((total + 255) / 256);
-    if (rblocks > 4096) rblocks = 4096;
-    if (d.dtype == ULTRAMEM_BF16) {
-        proj_kernel<__nv_bfloat16><<<grid, kThreads, 0, st>>>(d, p);
-        proj_reduce_kernel<__nv_bfloat16><<<rblocks, 256, 0, st>>>(d, p);
-    } else {
-        proj_kernel<float><<<grid, kThreads, 0, st>>>(d, p);
-        proj_reduce_kernel<float><<<rblocks, 256, 0, st>>>(d, p);
-    }
-    return cudaGetLastError();
+    const bool small = dot::small_tiles((int64_t)((d.d_out + 63) / 64) * ((d.B + 15) / 16) *
+                                        d.p_splits);
+    if (d.dtype == ULTRAMEM_BF16)
+        return small ? launch_proj_t<__nv_bfloat16, 1, 1>(d, p, st)
+                     : launch_proj_t<__nv_bfloat16, 2, 2>(d, p, st);
+    return small ? launch_proj_t<float, 1, 1>(d, p, st) : launch_proj_t<float, 2, 2>(d, p, st);
 }
 
 }  // namespace um

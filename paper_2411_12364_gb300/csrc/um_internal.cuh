@@ -2,8 +2,10 @@
 //
 // Every kernel receives the layer's dimensions (Dims) and the device pointers
 // it touches (Ptrs) by value.  Workspace layouts (all fp32 unless noted):
-//   q_part   [q_splits][A][B][H*D_k]   split-K partial sums of q = W_q x (the
-//                                      tensor path leaves the sum in split 0)
+//   q_part   [q_splits][A][B][H*D_k]   q = W_q x: the sum in split 0 (fp32 storage:
+//                                      also the fp64 sum, rounded, in split 1);
+//                                      before a query LayerNorm on CUDA cores,
+//                                      the split-K partial sums
 //   akey     [B][H][2][K] uint32       order-preserving key of the rank-1 score
 //                                      u^T S_row (axis 0) / t^T S_col (axis 1), Eq. 6
 //   sel_row  [B][H][m] int32           physical row of each selected slot
@@ -144,8 +146,9 @@ cudaError_t launch_dw_tc(const Dims &d, const CUtensorMap &g_t, const CUtensorMa
 cudaError_t launch_transpose_bf16(const void *src, void *dst, int rows, int cols,
                                   cudaStream_t st, int64_t ld_src = 0, int64_t ld_dst = 0);
 
-// x_f32: the token rows p.x are fp32 (the convolved input) whatever the storage type
-cudaError_t launch_query(const Dims &d, const Ptrs &p, bool x_f32, cudaStream_t st);
+// x_f32: the token rows p.x are fp32 (the convolved input) whatever the storage
+// type; reduce: the D_i splits are summed (see query_kernel), else stored
+cudaError_t launch_query(const Dims &d, const Ptrs &p, bool x_f32, bool reduce, cudaStream_t st);
 // Trick 4: the causal depthwise convolution of the call's tokens into p.xs
 // (three bf16 terms when `splits`, else fp32) and the conv state after them
 cudaError_t launch_query_conv(const Dims &d, const Ptrs &p, bool splits, cudaStream_t st);
@@ -165,6 +168,8 @@ cudaError_t launch_gather(const Dims &d, const Ptrs &p, cudaStream_t st);
 // the kernels reading sel_row / sel_p / sel_w serve.
 cudaError_t launch_gather_addresses(const Dims &d, const Ptrs &p, bool *taken, cudaStream_t st);
 cudaError_t launch_proj(const Dims &d, const Ptrs &p, cudaStream_t st);
+// kernel attributes of the CUDA-core query and scores (padded launches)
+cudaError_t configure_cuda_core();
 
 // The number-wise partitioned table (App. D): route slots to their rows'
 // owners (counts and cursor: [P] scratch), look rows up in a shard, and the
@@ -285,6 +290,8 @@ inline size_t spread_smem(size_t need, size_t static_bytes, int64_t ctas) {
     if (pad + static_bytes > kSmemPerCta) return need;
     return pad > need ? pad : need;
 }
+
+inline int64_t ctas_of(dim3 g) { return (int64_t)g.x * g.y * g.z; }
 
 // The static shared memory of kernel K (looked up once per kernel).
 template <auto K> size_t static_smem_of() {
@@ -468,6 +475,11 @@ struct Dot2 {
         c = __fadd_rn(c, o.c);
     }
     __device__ __forceinline__ float value() const { return __fadd_rn(s, c); }
+    // the sum where it may be infinite or NaN: s then is what plain sums give,
+    // and c, the sum of its rounding errors, is not a number
+    __device__ __forceinline__ float value_any() const {
+        return fabsf(s) < __int_as_float(0x7f800000) ? __fadd_rn(s, c) : s;
+    }
 };
 
 // Barrett's constant for reduction modulo M (P. Barrett, CRYPTO '86).
