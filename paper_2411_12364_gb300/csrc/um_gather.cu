@@ -362,6 +362,115 @@ __global__ void __launch_bounds__(THREADS, (sizeof(T) == 4 ? 512 : 1024) / THREA
     stamp_end(p.stamp);
 }
 
+// Long batches with a virtual expansion (bf16): one warp per (token, block),
+// four to a CTA, nothing shared between them.  A warp reads its token's slots,
+// keeps those of its block (ballots; slot order) in its own list, and sums
+// their rows, 8 in flight, a lane owning 16 bytes of each, so that the pooled
+// entries leave as 16-byte stores.  Against a CTA per token that sorts its
+// slots by block together: no barriers, no sums of several warps, and the SM
+// refills a warp at a time.  Bound: HBM.  Measured on GB300 (a call): decode_1m
+// with 2000 tokens and the query extras 157.0 -> 149.4 us (its gather 23 -> 16),
+// a lookup of 2048 tokens at mid_4m 84.0 -> 79.1, prefill_16k 1902 -> 1888
+// (376 us for 2.2 GB, 5.9 TB/s); with component cores, whose weights are
+// another dependent read, it is slower (180 -> 186 us at mid_4m with 1000).
+// HALVES: the block's rows as two sums, of the first and the second half.
+constexpr int kGWarps = 4;
+constexpr int kGSlots = 256;   // slots a token
+template <bool ADDR, bool HALVES>
+__global__ void __launch_bounds__(32 * kGWarps, 32 / kGWarps) gather_warp_kernel(Dims d, Ptrs p) {
+    extern __shared__ __align__(16) unsigned char gsm[];
+    constexpr int EPV = 8;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int hm = d.H * d.m, Dv = d.d_v;
+    const int64_t gw = (int64_t)blockIdx.x * kGWarps + warp;
+    const int64_t b = gw / d.E;
+    const int q = (int)(gw - b * d.E);
+    float4 *first_s = reinterpret_cast<float4 *>(gsm) + warp * 64;   // the first half's sums
+    int *row_s = reinterpret_cast<int *>(gsm + kGWarps * 1024) + warp * 2 * hm;   // its list
+    float *w_s = reinterpret_cast<float *>(row_s + hm);
+    pdl_wait();
+    stamp_begin(p.stamp);
+    pdl_trigger();
+    if (b < d.B) {   // warp-uniform
+        const int64_t base = b * hm;
+        int n = 0;
+        for (int j0 = 0; j0 < hm; j0 += 128) {   // 4 slots a lane: their loads together
+            int row[4], blk[4];
+            float w[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const int j = j0 + 32 * u + lane;
+                blk[u] = -1;
+                row[u] = 0;
+                w[u] = 0.f;
+                if (j < hm) {
+                    if constexpr (ADDR) {   // an invalid address weighs 0
+                        w[u] = p.w_in[base + j];
+                        if (!slot_of_address(d, p, p.idx_in[base + j], row[u], blk[u])) w[u] = 0.f;
+                    } else {
+                        row[u] = p.sel_row[base + j];
+                        blk[u] = p.sel_p[base + j];
+                        w[u] = p.sel_w[base + j];
+                    }
+                }
+            }
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const unsigned mine = __ballot_sync(0xffffffffu, blk[u] == q);
+                if (blk[u] == q) {
+                    const int at = n + __popc(mine & ((1u << lane) - 1u));
+                    row_s[at] = row[u];
+                    w_s[at] = w[u];
+                }
+                n += __popc(mine);
+            }
+        }
+        __syncwarp();
+        const bool active = lane * EPV < Dv;
+        const __nv_bfloat16 *V = static_cast<const __nv_bfloat16 *>(p.values) + lane * EPV;
+        float acc[EPV];
+        const int half = HALVES ? (n + 1) / 2 : 0;
+#pragma unroll 1
+        for (int part = HALVES ? 0 : 1; part < 2; ++part) {
+            const int lo = part ? half : 0, hi = part ? n : half;
+#pragma unroll
+            for (int c = 0; c < EPV; ++c) acc[c] = 0.f;
+#pragma unroll 1
+            for (int j0 = lo; j0 < hi; j0 += kUnroll) {
+                uint4 val[kUnroll];
+                float wu[kUnroll];
+#pragma unroll
+                for (int u = 0; u < kUnroll; ++u) {
+                    const int j = j0 + u;
+                    const bool ok = j < hi;
+                    wu[u] = ok ? w_s[j] : 0.f;
+                    val[u] = (ok && active) ? ld_stream(V + (int64_t)row_s[j] * Dv)
+                                            : make_uint4(0, 0, 0, 0);
+                }
+#pragma unroll
+                for (int u = 0; u < kUnroll; ++u) {
+                    float f[EPV];
+                    unpack<__nv_bfloat16>(val[u], f);
+#pragma unroll
+                    for (int c = 0; c < EPV; ++c) acc[c] = fmaf(wu[u], f[c], acc[c]);
+                }
+            }
+            if (HALVES && !part) {
+                first_s[lane] = make_float4(acc[0], acc[1], acc[2], acc[3]);
+                first_s[32 + lane] = make_float4(acc[4], acc[5], acc[6], acc[7]);
+            }
+        }
+        if (HALVES) {
+            const float4 x = first_s[lane], y = first_s[32 + lane];
+            const float h[EPV] = {x.x, x.y, x.z, x.w, y.x, y.y, y.z, y.w};
+#pragma unroll
+            for (int c = 0; c < EPV; ++c) acc[c] = h[c] + acc[c];
+        }
+        if (active) store_pooled8(d, p, b, q * Dv + lane * EPV, acc);
+    }
+    stamp_end(p.stamp);
+}
+
 // Shared-memory-accumulating gather for any E and row width (A: the
 // accumulator, fp64 for fp32 storage while [kWarps][E][D_v] of it fits).
 template <typename T, typename A>
@@ -551,6 +660,20 @@ static cudaError_t launch_bucket(const Dims &d, const Ptrs &p, bool *taken, cuda
     constexpr int epv = 16 / (int)sizeof(T);
     *taken = false;
     if (d.d_v % epv || d.E > kBMaxE) return cudaSuccess;
+    if constexpr (!std::is_same<T, float>::value) {
+        // from 305 tokens on (the 512-thread CTAs' limit), blocks to spread over
+        if (d.B > 2 * 152 && d.E > 1 && d.nc == 1 && d.H * d.m <= kGSlots &&
+            d.d_v / epv <= 32) {
+            *taken = true;
+            const int64_t warps = (int64_t)d.B * d.E;
+            const int grid = (int)((warps + kGWarps - 1) / kGWarps);
+            const size_t smem = (size_t)kGWarps * (1024 + 8 * (size_t)d.H * d.m);
+            return d.E == 4 ? launch_kernel(d.pdl, gather_warp_kernel<ADDR, true>, grid,
+                                            32 * kGWarps, smem, st, d, p)
+                            : launch_kernel(d.pdl, gather_warp_kernel<ADDR, false>, grid,
+                                            32 * kGWarps, smem, st, d, p);
+        }
+    }
     if (d.d_v / epv <= 32) return launch_bucket_v<T, ADDR, 1>(d, p, taken, st);
     if constexpr (std::is_same<T, float>::value)
         if (d.d_v / epv <= 64) return launch_bucket_v<T, ADDR, 2>(d, p, taken, st);

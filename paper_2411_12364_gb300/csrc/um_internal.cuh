@@ -443,6 +443,57 @@ __device__ __forceinline__ void store_pooled(const Dims &d, const Ptrs &p, int64
     }
 }
 
+// Eight consecutive pooled values (bf16 storage; i a multiple of 8) as 16-byte
+// stores.
+__device__ __forceinline__ void store_pooled8(const Dims &d, const Ptrs &p, int64_t b, int i,
+                                              const float (&v)[8]) {
+    const int EDv = d.E * d.d_v;
+    auto put = [](__nv_bfloat16 *dst, const float (&x)[8]) {
+        uint32_t u[4];
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+            const __nv_bfloat162 t = __floats2bfloat162_rn(x[2 * c], x[2 * c + 1]);
+            u[c] = *reinterpret_cast<const uint32_t *>(&t);
+        }
+        *reinterpret_cast<uint4 *>(dst) = make_uint4(u[0], u[1], u[2], u[3]);
+    };
+    if (p.acc_bf) {
+        __nv_bfloat16 *dst = p.acc_bf + b * p.acc_terms * EDv + i;
+        float t[8], r[8];
+        if (p.acc_terms == 3) {
+            bool fin[8];
+#pragma unroll
+            for (int c = 0; c < 8; ++c) {
+                fin[c] = fabsf(v[c]) < __int_as_float(0x7f800000);
+                t[c] = fin[c] ? cut_bf16(v[c]) : v[c];
+                r[c] = fin[c] ? v[c] - t[c] : 0.f;
+            }
+            put(dst, t);
+#pragma unroll
+            for (int c = 0; c < 8; ++c) {
+                t[c] = cut_bf16(r[c]);
+                r[c] -= t[c];
+            }
+            put(dst + EDv, t);
+            put(dst + 2 * EDv, r);
+        } else {
+#pragma unroll
+            for (int c = 0; c < 8; ++c)
+                r[c] = v[c] - __bfloat162float(__float2bfloat16_rn(v[c]));
+            put(dst, v);
+            put(dst + EDv, r);
+        }
+    } else if (d.has_proj) {
+        float4 *dst = reinterpret_cast<float4 *>(p.acc + b * EDv + i);
+        dst[0] = make_float4(v[0], v[1], v[2], v[3]);
+        dst[1] = make_float4(v[4], v[5], v[6], v[7]);
+    } else {
+        __nv_bfloat16 *dst = static_cast<__nv_bfloat16 *>(p.out) + b * d.d_v + i;
+#pragma unroll
+        for (int c = 0; c < 8; ++c) dst[c] = __float2bfloat16_rn(v[c]);
+    }
+}
+
 // ---- fp32 storage: dot products to the working precision ---------------
 // The fp32 mode promises outputs within 1e-4 of the exact result element by
 // element (down to 1e-3 of a row's largest entry), which plain fp32

@@ -1,6 +1,7 @@
 """GPU parity of the lookup-reduce on given slots (S7-S9, Eq. 14-15) where its
 dispatch changes: the gather that reads addresses (512 threads up to 304
-tokens, 256 above, the slots kernel for more slots than those serve) and the
+tokens, above a warp per block or, with component cores, 256 threads; the
+slots kernel for more slots than those serve) and the
 tensor-core projection with the pooled rows as three bf16 terms (split over
 its inner dimension at small batches, persistent at long ones)."""
 import numpy as np
@@ -33,7 +34,9 @@ CASES = [
     (dict(d_v=256, d_out=512, heads=4, topk=16, topm=128), 304, 2),   # 512 slots a token
     (dict(d_v=256, d_out=512, heads=4, topk=16, topm=64), 305, 2),    # 256 threads
     (dict(d_v=256, d_out=512, heads=4, topk=16, topm=65), 305, 3),    # 260 slots: slots kernel
-    (dict(d_v=72, d_out=264, expand_e=9, n=11), 700, 3),       # E > 8; K blocks across the terms
+    (dict(d_v=72, d_out=264, expand_e=9, n=11), 700, 2),       # a warp per block; ragged K blocks
+    (dict(d_v=256, d_out=512, heads=2, topk=16, topm=70), 305, 2),    # 140 slots: two rounds
+    (dict(d_v=128, d_out=512, cores=2, heads=4), 310, 2),      # cores: a CTA per token
     (dict(d_v=256, d_out=2048, topk=16, topm=16), 3000, 2),    # more tiles than SMs
 ]
 
