@@ -503,7 +503,7 @@ ultramem_status run_tensor(ultramem_layer *L, const Dims &d, Ptrs p, cudaStream_
     if (!um::tc_encode(&mp.qs, L->ws.qs, 3ull * c.d_k, (uint64_t)Bmax, 2ull * d.H,
                        (uint32_t)nt1, 3) ||
         !um::tc_encode(&mp.acc, L->ws.acc_bf, 2ull * d.E * d.d_v, (uint64_t)Bmax, 1,
-                       (uint32_t)d.p_ntile, 2))
+                       um::proj_token_box(d), 2))
         return ULTRAMEM_ECUDA;
     // the projection reads the pooled rows as two bf16 terms hi + lo
     p.acc_bf = c.has_proj ? L->ws.acc_bf : nullptr;
@@ -599,7 +599,7 @@ ultramem_status pool_and_project(ultramem_layer *L, const Dims &d0, Ptrs p,
     CUtensorMap acc_map;
     const bool tc = L->tc && d.has_proj && macs >= kTcLookupMacs &&
                     um::tc_encode(&acc_map, L->ws.acc_bf, 3ull * d.E * d.d_v,
-                                  (uint64_t)L->cfg.max_tokens, 1, (uint32_t)d.p_ntile, 2);
+                                  (uint64_t)L->cfg.max_tokens, 1, um::proj_token_box(d), 2);
     if (tc) {
         p.acc_bf = L->ws.acc_bf;
         p.acc_terms = 3;

@@ -130,6 +130,8 @@ cudaError_t configure_small();
 // instead of x itself
 cudaError_t launch_query_small(const Dims &d, const Ptrs &p, __nv_bfloat16 *qs, int Bmax,
                                bool x_f32, bool write_qs, bool pdl, cudaStream_t st);
+// tokens a TMA box of the projection's map acc covers
+uint32_t proj_token_box(const Dims &d);
 // acc_terms: bf16 terms of the pooled rows (map acc over [B][acc_terms E D_v])
 cudaError_t launch_proj_tc(const Dims &d, const Ptrs &p, const TcMaps &mp, int acc_terms,
                            cudaStream_t st);

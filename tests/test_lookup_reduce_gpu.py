@@ -31,6 +31,8 @@ CASES = [
     (dict(d_v=256, d_out=1024, heads=1), 1, 2),                # one token, split
     (dict(d_v=256, d_out=1000), 37, 2),                        # ragged rows of W_p^T
     (dict(d_v=128, d_out=520, cores=2), 130, 2),               # two weights a slot
+    (dict(d_v=128, d_out=523), 200, 2),                        # output rows off 16 bytes
+    (dict(d_v=64, d_out=4096), 1000, 2),                       # 256-output tiles, one wave
     (dict(d_v=256, d_out=512, heads=4, topk=16, topm=128), 304, 2),   # 512 slots a token
     (dict(d_v=256, d_out=512, heads=4, topk=16, topm=64), 305, 2),    # 256 threads
     (dict(d_v=256, d_out=512, heads=4, topk=16, topm=65), 305, 3),    # 260 slots: slots kernel
