@@ -20,21 +20,23 @@ constexpr int kK = 32;   // k staged at once
 // One pair of outputs' Dot2 sums (Dot2's steps, packed).  add takes the A
 // value in both halves as it is and negated: with np = -(a b) rounded, every
 // step of Dot2 is one packed instruction, and each half rounds as there.
+// Products go into multiply-adds only: the compiler fuses a packed product
+// with a packed sum that takes it, although both round on their own.
 struct Dot2x2 {
     using Elem = float4;   // an A value as it is staged: (a, a, -a, -a)
     static __device__ __forceinline__ Elem stage(float a) { return make_float4(a, a, -a, -a); }
     f2 s, c;
     __device__ __forceinline__ Dot2x2() : s(0ull), c(0ull) {}
     __device__ __forceinline__ void add(f2 a, f2 na, f2 b) {
-        const f2 one = 0xbf800000bf800000ull;        // (-1, -1)
+        const f2 m1 = 0xbf800000bf800000ull;               // (-1, -1)
         const f2 np = mul2(na, b);
-        const f2 pe = fma2(a, b, np);                // a b - p, exact
-        const f2 t = fma2(np, one, s);               // s + p
-        const f2 z = fma2(s, one, t);                // t - s
-        const f2 v = fma2(fma2(z, one, t), one, s);  // s - (t - z)
-        const f2 w = add2(np, z);                    // -(p - z)
+        const f2 pe = fma2(a, b, np);                      // a b - p, exact
+        const f2 t = fma2(np, m1, s);                      // s + p
+        const f2 zn = fma2(t, m1, s);                      // -z = s - t
+        const f2 v = fma2(add2(t, zn), m1, s);             // s - (t - z)
+        const f2 w = fma2(np, m1, zn);                     // p - z
         s = t;
-        c = add2(c, fma2(w, one, v));
+        c = add2(c, add2(v, w));
         c = add2(c, pe);
     }
     __device__ __forceinline__ float2 value() const { return unpack2(add2(s, c)); }

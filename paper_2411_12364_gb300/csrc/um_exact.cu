@@ -9,20 +9,24 @@
 //      R[i] = S_row[:,i]^T C and S_col[:,j] (product keys: s_row[i] and
 //      s_col[j]), so that g(i,j) = R[i] . S_col[j] (or the sum) with the
 //      forward's own arithmetic;
-//   2. one pass over the grid: a thread holds four columns' S_col in
+//   2. rows that cannot hold a winner are dropped: a score is at most
+//      |R[i]| |S_col[j]|, so from a bound tau0 <= the m-th largest score, taken
+//      by steps 3 and 4 over the 64 or so longest rows alone, every row with
+//      |R[i]| max_j |S_col[j]| < tau0 goes (a Gaussian grid of 2048 rows keeps
+//      some tens of them);
+//   3. one pass over the rows left: a thread holds four columns' S_col in
 //      registers, streams the rows (broadcast from shared memory, two rows a
 //      packed fp32 instruction) and keeps the largest score of each of 8
 //      shares of its pairs, so the grid falls into 4096 groups;
-//   3. tau, at most the m-th largest of the group maxima (m distinct groups
+//   4. tau, at most the m-th largest of the group maxima (m distinct groups
 //      reach it, so the top m is >= tau); only the groups whose maximum
-//      reaches tau (about m of 4096) are scored again, a warp per group, and
-//      their scores >= tau, as (key, ~v) composites, go to a list;
-//   4. ranks by (score desc, address asc).
-// The one full pass is bound by the fp32 pipe: two operations a pair at rank
-// 2, 27 us for decode_1m's 64 tokens x 2 heads x 2048^2 pairs at 152 SMs x
-// 128 lanes x 2.07 GHz.  Measured there: 9146 us with the radix select below
-// for every grid (9 passes over the pairs, a histogram atomic per pair and
-// pass, a warp per key in step 1) -> 179 us.
+//      reaches tau are scored again, a warp per group, and their scores >=
+//      tau, as (key, ~v) composites, go to a list;
+//   5. ranks by (score desc, address asc).
+// Measured on GB300, decode_1m's 64 tokens x 2 heads: 9146 us with the radix
+// select below for every grid (9 passes over the pairs, a histogram atomic per
+// pair and pass), 179 us with steps 3 to 5 over every row (the pass alone is
+// 27 us of fp32 work) and a warp per 16 keys in step 1, 84 us now.
 //
 // When the list overflows (heavy ties) or a chunk score is not finite (its
 // score may be a NaN, which the maxima would not see), the CTA takes an
@@ -54,8 +58,9 @@ constexpr int kBoundBits = 20;    // leading key bits that tau is searched in
 constexpr int kMaxShares = 16;
 
 struct ExactShared {
-    int hist[256];        // the radix select's; before it, entry st counts the group
-                          // maxima at or above the trial bound of step st
+    int hist[256];        // the radix select's; before it, the bound searches' counts
+    int scan[kWarps];
+    uint32_t smax;        // the largest |S_col|^2 (product keys: key of S_col)
     int count;            // listed candidates (may exceed the list)
     uint32_t prefix;      // key bits fixed so far
     int need;             // how many of the remaining keys are still to take
@@ -69,14 +74,26 @@ constexpr size_t kStatic = (sizeof(ExactShared) + 15) & ~size_t(15);
 // Dynamic shared memory: the candidate list (the core in it while the chunk
 // scores are computed), R [r][rows] and S_col [r][K] by rank (rows and K
 // padded to 16 bytes), the query [2][D_k].
+// With room for it, a stage: 32 keys x 32 elements a warp for step 1, then the
+// seed rows and the kept rows' numbers of step 2.
 __host__ __device__ inline int pad4(int x) { return (x + 3) & ~3; }
+constexpr int kSeedRows = 64, kSeedMax = 128;
+template <typename T> __host__ __device__ constexpr int stage_pitch() {
+    return 32 * (int)sizeof(T) + 16;   // bytes a key: its 16-byte reads miss no bank twice
+}
+inline size_t stage_bytes_of(const Dims &d, int rows) {
+    const size_t keys = (size_t)kWarps * 32 *
+                        (d.dtype == ULTRAMEM_F32 ? stage_pitch<float>() : stage_pitch<uint16_t>());
+    const size_t prune = 4 * (size_t)kSeedMax * d.r + ((2 * (size_t)rows + 15) & ~size_t(15));
+    return keys > prune ? keys : prune;
+}
 inline size_t exact_smem(const Dims &d, int rows, int list) {
     return 8 * (size_t)list + sizeof(float) * ((size_t)d.r * (pad4(rows) + pad4(d.K)) + 2 * d.d_k);
 }
 // The list's length: as long as fits, at most kListMax, at least kMaxM.
-inline int list_len(const Dims &d, int rows) {
+inline int list_len(const Dims &d, int rows, size_t stage) {
     int n = kListMax;
-    while (n > kMaxM && exact_smem(d, rows, n) + kStatic > kSmemPerCta) n -= 128;
+    while (n > kMaxM && exact_smem(d, rows, n) + stage + kStatic > kSmemPerCta) n -= 128;
     return n;
 }
 // Shares of rows per (token, head): about one CTA per SM, at most K / m (so
@@ -197,8 +214,12 @@ __device__ int pick_bin_from_bottom(const int *hist, int &need) {
 // fewer than the share holds never) by a radix select of the m-th largest
 // key over the scores, recomputed each pass, with one shared atomic per
 // distinct bin and warp.  Whole block; ends with a barrier.
-__device__ __noinline__ void radix_top_m(Grid gd, u64 *list, int i0, int nr, int K, int m,
-                                         ExactShared &sh) {
+__device__ __noinline__ void radix_top_m(Grid gd, u64 *list, const uint16_t *map, int i0, int nr,
+                                         int K, int m, ExactShared &sh) {
+    // the address of (row i, column j); map: the numbers of the rows kept, or null
+    auto addr = [&](int i, int j) {
+        return (uint32_t)(i0 + (map ? (int)map[i] : i)) * (uint32_t)K + (uint32_t)j;
+    };
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int64_t total = (int64_t)nr * K;
     const int64_t iters = (total + kThreads - 1) / kThreads;
@@ -254,7 +275,7 @@ __device__ __noinline__ void radix_top_m(Grid gd, u64 *list, int i0, int nr, int
             for (int64_t it = 0; it < iters; ++it) {
                 int bin = 256;
                 if (i < nr && f2ord(gd.score(i, j)) == thr) {
-                    const uint32_t v = (uint32_t)(i0 + i) * (uint32_t)K + (uint32_t)j;
+                    const uint32_t v = addr(i, j);
                     if ((v & hi_mask) == (pre & hi_mask)) bin = (v >> shift) & 255;
                 }
                 warp_hist(sh.hist, bin);
@@ -284,7 +305,7 @@ __device__ __noinline__ void radix_top_m(Grid gd, u64 *list, int i0, int nr, int
             uint32_t key = 0, v = 0;
             if (i < nr) {
                 key = f2ord(gd.score(i, j));
-                v = (uint32_t)(i0 + i) * (uint32_t)K + (uint32_t)j;
+                v = addr(i, j);
                 take = key > thr || (key == thr && v <= vcut);
             }
             const unsigned bal = __ballot_sync(kFull, take);
@@ -348,11 +369,226 @@ __device__ __forceinline__ void chunk_scores(const T *rows, int n, const float *
     }
 }
 
+// The chunk scores of `n` keys against q, a lane per key: a warp's 32 rows come
+// in 32 elements at a time through its stage (16-byte loads of whole sectors,
+// the next ones on their way meanwhile), and a lane adds up its key's
+// products by the same tree as chunk_scores' 32 lanes: 32 partial sums over
+// the elements l, l + 32, ... of a chunk, packed in pairs, then halves.
+// put(key, s): the lane's chunk sums.  dk % 32 == 0, rows 16-byte aligned.
+template <typename T, int RP, class Put>
+__device__ __forceinline__ void chunk_scores_staged(const T *rows, int n, const float *q, int D,
+                                                    int dk, int r, unsigned char *stage, Put put) {
+    constexpr int VB = 32 * (int)sizeof(T) / 16, PITCH = stage_pitch<T>();
+    constexpr int EPV = 16 / (int)sizeof(T);
+    constexpr f2 kMinus1 = 0xbf800000bf800000ull;   // (-1, -1)
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    unsigned char *mine = stage + warp * 32 * PITCH;
+    const int steps = D / 32;
+    for (int k0 = warp * 32; k0 < n; k0 += kWarps * 32) {
+        uint4 buf[VB];
+        auto fetch = [&](int st) {
+#pragma unroll
+            for (int i = 0; i < VB; ++i) {
+                const int e = i * 32 + lane, key = min(k0 + e / VB, n - 1);
+                buf[i] = *reinterpret_cast<const uint4 *>(rows + (int64_t)key * D + 32 * st +
+                                                          e % VB * EPV);
+            }
+        };
+        float s[RP];
+#pragma unroll
+        for (int a = 0; a < RP; ++a) s[a] = 0.f;
+        f2 v[16];
+        int al = 0, left = dk / 32;   // the chunk, and its steps to go
+        fetch(0);
+#pragma unroll 1
+        for (int st = 0; st < steps; ++st) {
+            __syncwarp();   // the previous elements have been read
+#pragma unroll
+            for (int i = 0; i < VB; ++i) {
+                const int e = i * 32 + lane;
+                *reinterpret_cast<uint4 *>(mine + e / VB * PITCH + e % VB * 16) = buf[i];
+            }
+            __syncwarp();
+            if (st + 1 < steps) fetch(st + 1);
+            if (left == dk / 32)   // uniform: a chunk starts
+#pragma unroll
+                for (int j = 0; j < 16; ++j) v[j] = 0ull;
+#pragma unroll
+            for (int i = 0; i < VB; ++i) {
+                const uint4 x = *reinterpret_cast<const uint4 *>(mine + lane * PITCH + i * 16);
+                const ulonglong2 *qq =
+                    reinterpret_cast<const ulonglong2 *>(q + 32 * st + i * EPV);
+                const uint32_t w[4] = {x.x, x.y, x.z, x.w};
+                f2 xe[EPV / 2];
+#pragma unroll
+                for (int c = 0; c < EPV / 2; ++c) {
+                    if constexpr (sizeof(T) == 2)
+                        xe[c] = pack2(__uint_as_float(w[c] << 16),
+                                      __uint_as_float(w[c] & 0xffff0000u));
+                    else
+                        xe[c] = pack2(__uint_as_float(w[2 * c]), __uint_as_float(w[2 * c + 1]));
+                }
+#pragma unroll
+                for (int c = 0; c < EPV / 2; c += 2) {
+                    const ulonglong2 q2 = qq[c / 2];
+                    const int at = i * (EPV / 2) + c;
+                    // v holds the negated sums: a product of -1 keeps the
+                    // compiler from fusing the product into the sum
+                    v[at] = fma2(mul2(xe[c], q2.x), kMinus1, v[at]);
+                    v[at + 1] = fma2(mul2(xe[c + 1], q2.y), kMinus1, v[at + 1]);
+                }
+            }
+            if (--left == 0) {
+#pragma unroll
+                for (int half = 8; half > 0; half >>= 1)
+#pragma unroll
+                    for (int j = 0; j < half; ++j) v[j] = add2(v[j], v[j + half]);
+                const float2 x = unpack2(v[0]);
+                const float sum = -__fadd_rn(x.x, x.y);
+#pragma unroll
+                for (int a = 0; a < RP; ++a)
+                    if (a == al) s[a] = sum;
+                ++al;
+                left = dk / 32;
+            }
+        }
+        if (k0 + lane < n) put(k0 + lane, s);
+    }
+}
+
+// The largest value with zero low bits (`bits` leading ones of 32 decided)
+// that at least `need` of the block's keys reach; each(f) calls f(key) for the
+// thread's keys.  cnt: `bits` counters, zero.  Whole block.
+template <class Each>
+__device__ __forceinline__ uint32_t block_bound(int need, int bits, int *cnt, Each each) {
+    uint32_t T = 0u;
+#pragma unroll 1
+    for (int st = 0; st < bits; ++st) {
+        const uint32_t c = T | (0x80000000u >> st);
+        int n = 0;
+        each([&](uint32_t key) { n += key >= c; });
+        n = __reduce_add_sync(kFull, n);
+        if ((threadIdx.x & 31) == 0 && n) atomicAdd(&cnt[st], n);
+        __syncthreads();
+        if (cnt[st] >= need) T = c;
+    }
+    return T;
+}
+
+// Exclusive prefix sum of one int per thread over the block, and the total.
+__device__ __forceinline__ int block_scan(int v, ExactShared &sh, int *total) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    int incl = v;
+#pragma unroll
+    for (int off = 1; off < 32; off <<= 1) {
+        const int y = __shfl_up_sync(kFull, incl, off);
+        if (lane >= off) incl += y;
+    }
+    __syncthreads();   // the previous scan's sums have been read
+    if (lane == 31) sh.scan[warp] = incl;
+    __syncthreads();
+    int before = 0, all = 0;
+    for (int w = 0; w < kWarps; ++w) {
+        const int x = sh.scan[w];
+        before += w < warp ? x : 0;
+        all += x;
+    }
+    *total = all;
+    return before + incl - v;
+}
+
+__device__ __forceinline__ float max3(float a, float b, float c) {
+    float m;
+    asm("max.f32 %0, %1, %2, %3;" : "=f"(m) : "f"(a), "f"(b), "f"(c));
+    return m;
+}
+
+// A thread's part of a pass: column group cg of a block of columns takes kCols
+// consecutive ones; when the columns are fewer than the threads hold, rs_n
+// threads share a column group and take every rs_n-th quad of rows.  Part q
+// of a thread is the q-th eighth of its `mine` quads.
+struct PassShape {
+    int rs_n, rs, cg, mine;
+    bool busy;
+    __device__ __forceinline__ PassShape(int nr, int K) {
+        const int cgs = min(kThreads, (K + kCols - 1) / kCols);
+        rs_n = kThreads / cgs;
+        rs = threadIdx.x / cgs;
+        cg = threadIdx.x - rs * cgs;
+        busy = rs < rs_n;
+        const int quads = pad4(nr) >> 2;
+        mine = busy && quads > rs ? (quads - rs + rs_n - 1) / rs_n : 0;
+    }
+    __device__ __forceinline__ int lo(int q) const { return mine * q / kParts; }
+};
+
+// The largest score of each of the thread's parts, as keys (0: an empty part),
+// over the rows R [r][Rp] (the last quad padded by repeats) and all columns.
+template <int RP, bool PKM>
+__device__ __forceinline__ void group_maxima(const float *R, int Rp, const float *S, int Sp, int r,
+                                             int K, const PassShape &ps, uint32_t (&gk)[kParts]) {
+    float gm[kParts];
+#pragma unroll
+    for (int q = 0; q < kParts; ++q) gm[q] = -INFINITY;
+    for (int j0 = kCols * ps.cg; ps.busy && j0 < K; j0 += kCols * kThreads) {
+        // the columns' S, each in both halves; a missing column repeats the
+        // thread's first (which changes no maximum)
+        f2 sc[RP][kCols];
+#pragma unroll
+        for (int be = 0; be < RP; ++be)
+#pragma unroll
+            for (int c = 0; c < kCols; ++c) {
+                const float v = be < r ? S[be * Sp + (j0 + c < K ? j0 + c : j0)] : 0.f;
+                sc[be][c] = pack2(v, v);
+            }
+#pragma unroll
+        for (int q = 0; q < kParts; ++q) {
+            const int hi = ps.lo(q + 1);
+            float mx0 = gm[q], mx1 = -INFINITY;
+#pragma unroll 2
+            for (int t = ps.lo(q); t < hi; ++t) {
+                const int i = 4 * (ps.rs + t * ps.rs_n);
+                f2 ra[RP][2];   // rows i, i + 1 and i + 2, i + 3
+#pragma unroll
+                for (int be = 0; be < RP; ++be) {
+                    ulonglong2 v = make_ulonglong2(0ull, 0ull);
+                    if (be < r) v = *reinterpret_cast<const ulonglong2 *>(R + be * Rp + i);
+                    ra[be][0] = v.x;
+                    ra[be][1] = v.y;
+                }
+#pragma unroll
+                for (int c = 0; c < kCols; ++c) {
+                    f2 g[2];
+#pragma unroll
+                    for (int u = 0; u < 2; ++u) {
+                        if (PKM) {
+                            g[u] = add2(ra[0][u], sc[0][c]);
+                        } else {
+                            g[u] = mul2(ra[0][u], sc[0][c]);
+#pragma unroll
+                            for (int be = 1; be < RP; ++be)
+                                g[u] = fma2(ra[be][u], sc[be][c], g[u]);
+                        }
+                    }
+                    const float2 x = unpack2(g[0]), y = unpack2(g[1]);
+                    mx0 = max3(mx0, x.x, x.y);
+                    mx1 = max3(mx1, y.x, y.y);
+                }
+            }
+            gm[q] = fmaxf(mx0, mx1);
+        }
+    }
+#pragma unroll
+    for (int q = 0; q < kParts; ++q)
+        gk[q] = ps.lo(q + 1) > ps.lo(q) && kCols * ps.cg < K ? f2ord(gm[q]) : 0u;
+}
+
 // RP: the rank rounded up to 1, 2, 4 or 8 (missing chunks are zeros, which
 // leave the sums as they are).
 template <typename T, int RP, bool PKM>
 __global__ void __launch_bounds__(kThreads, 1)
-    exact_kernel(Dims d, Ptrs p, int shares, int list_n, int64_t *idx_out, float *w_out) {
+    exact_kernel(Dims d, Ptrs p, int shares, int list_n, int staged, int64_t *idx_out,
+                 float *w_out) {
     extern __shared__ __align__(16) unsigned char exact_raw[];
     __shared__ ExactShared sh;
     const int pair = blockIdx.x / shares, share = blockIdx.x - pair * shares;
@@ -361,12 +597,14 @@ __global__ void __launch_bounds__(kThreads, 1)
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     // rows [i0, i0 + nr) of the grid; every share's space is the first one's
     const int per = (K + shares - 1) / shares;
-    const int i0 = share * per, nr = min(per, K - i0);
+    const int i0 = share * per;
+    int nr = min(per, K - i0);
     const int Rp = pad4(per), Sp = pad4(K);
     u64 *list = reinterpret_cast<u64 *>(exact_raw);
     float *core = reinterpret_cast<float *>(list);
     float *R = reinterpret_cast<float *>(list + list_n), *S = R + (size_t)r * Rp,
           *qv = S + (size_t)r * Sp;
+    unsigned char *stage = reinterpret_cast<unsigned char *>(qv + 2 * pad4(D));
     pdl_wait();
     pdl_trigger();
 
@@ -381,12 +619,13 @@ __global__ void __launch_bounds__(kThreads, 1)
         qv[e] = q;
     }
     if (threadIdx.x < r * r) core[threadIdx.x] = p.core[(int64_t)h * r * r + threadIdx.x];
-    if (threadIdx.x < kBoundBits) sh.hist[threadIdx.x] = 0;
+    if (threadIdx.x < 256) sh.hist[threadIdx.x] = 0;
     if (threadIdx.x == 0) {
         sh.count = 0;
         sh.prefix = 0;
         sh.need = m;
         sh.general = 0;
+        sh.smax = 0u;
     }
     __syncthreads();
 
@@ -402,7 +641,23 @@ __global__ void __launch_bounds__(kThreads, 1)
         if (j < K && be < r) S[be * Sp + j] = v;
         if (j < K && be < r && !(fabsf(v) < INFINITY)) odd = true;
     };
-    if (dk % 32 == 0) {
+    if (staged && dk % 32 == 0) {
+        chunk_scores_staged<T, RP>(krow, nr, qv, D, dk, r, stage, [&](int i, const float (&v)[RP]) {
+#pragma unroll
+            for (int be = 0; be < RP; ++be) {
+                float acc = 0.f;
+#pragma unroll
+                for (int a = 0; a < RP; ++a)
+                    if (a < r && be < r) acc = fmaf(v[a], core[a * r + be], acc);
+                put_r(i, be, acc);
+            }
+        });
+        chunk_scores_staged<T, RP>(kcol, K, qv + D, D, dk, r, stage,
+                                   [&](int j, const float (&v)[RP]) {
+#pragma unroll
+                                       for (int be = 0; be < RP; ++be) put_s(j, be, v[be]);
+                                   });
+    } else if (dk % 32 == 0) {
         chunk_scores<T, RP>(krow, nr, qv, D, dk, r, [&](int i, int be, float v, int l0) {
             float acc = 0.f;
 #pragma unroll
@@ -451,118 +706,133 @@ __global__ void __launch_bounds__(kThreads, 1)
     if (odd) sh.general = 1;
     __syncthreads();
     // the rows padding the last quad repeat the last row (their scores change
-    // no maximum)
-    if (threadIdx.x < 4 * r) {
-        const int be = threadIdx.x >> 2, i = nr + (threadIdx.x & 3);
-        if (i < pad4(nr)) R[be * Rp + i] = R[be * Rp + nr - 1];
-    }
-    __syncthreads();
+    // no maximum); ends with a barrier
+    auto pad_rows = [&](float *rows, int pitch, int n) {
+        if (threadIdx.x < 4 * r) {
+            const int be = threadIdx.x >> 2, i = n + (threadIdx.x & 3);
+            if (i < pad4(n)) rows[be * pitch + i] = rows[be * pitch + n - 1];
+        }
+        __syncthreads();
+    };
+    pad_rows(R, Rp, nr);
 
-    const Grid gd{R, S, Rp, Sp, r, d.pkm};
     bool general = sh.general != 0;   // uniform
-    if (!general) {
-        // 2. group maxima.  Column group cg of a block of columns takes 4
-        // consecutive ones; when the columns are fewer than the threads
-        // hold, `rs_n` threads share a column group and take every rs_n-th
-        // quad of rows.  Part q of a thread is the q-th eighth of its quads.
-        const int cgs = min(kThreads, (K + kCols - 1) / kCols);
-        const int rs_n = kThreads / cgs;
-        const int rs = threadIdx.x / cgs, cg = threadIdx.x - rs * cgs;
-        const bool busy = rs < rs_n;
-        const int quads = pad4(nr) >> 2, mine = busy && quads > rs ? (quads - rs + rs_n - 1) / rs_n : 0;
-        float gm[kParts];
-#pragma unroll
-        for (int q = 0; q < kParts; ++q) gm[q] = -INFINITY;
-        for (int j0 = kCols * cg; busy && j0 < K; j0 += kCols * kThreads) {
-            // the columns' S, each in both halves; a missing column repeats
-            // the thread's first (which changes no maximum)
-            f2 sc[RP][kCols];
-#pragma unroll
-            for (int be = 0; be < RP; ++be)
-#pragma unroll
-                for (int c = 0; c < kCols; ++c) {
-                    const float v = be < r ? S[be * Sp + (j0 + c < K ? j0 + c : j0)] : 0.f;
-                    sc[be][c] = pack2(v, v);
-                }
-#pragma unroll
-            for (int q = 0; q < kParts; ++q) {
-                const int lo = mine * q / kParts, hi = mine * (q + 1) / kParts;
-                float mx0 = gm[q], mx1 = -INFINITY;
-#pragma unroll 2
-                for (int t = lo; t < hi; ++t) {
-                    const int i = 4 * (rs + t * rs_n);
-                    f2 ra[RP][2];   // rows i, i + 1 and i + 2, i + 3
-#pragma unroll
-                    for (int be = 0; be < RP; ++be) {
-                        ulonglong2 v = make_ulonglong2(0ull, 0ull);
-                        if (be < r) v = *reinterpret_cast<const ulonglong2 *>(R + be * Rp + i);
-                        ra[be][0] = v.x;
-                        ra[be][1] = v.y;
-                    }
-#pragma unroll
-                    for (int c = 0; c < kCols; ++c) {
-                        f2 g[2];
-#pragma unroll
-                        for (int u = 0; u < 2; ++u) {
-                            if (PKM) {
-                                g[u] = add2(ra[0][u], sc[0][c]);
-                            } else {
-                                g[u] = mul2(ra[0][u], sc[0][c]);
-#pragma unroll
-                                for (int be = 1; be < RP; ++be)
-                                    g[u] = fma2(ra[be][u], sc[be][c], g[u]);
-                            }
-                        }
-                        const float2 x = unpack2(g[0]), y = unpack2(g[1]);
-                        mx0 = fmaxf(mx0, fmaxf(x.x, x.y));
-                        mx1 = fmaxf(mx1, fmaxf(y.x, y.y));
-                    }
-                }
-                gm[q] = fmaxf(mx0, mx1);
+    const uint16_t *map = nullptr;    // the kept rows' numbers
+    if (!general && staged && nr >= 4 * kSeedMax) {
+        // 2. |R[i]|^2 (product keys: R[i]) as a key; pads keep underflowed
+        // squares from pruning
+        constexpr float kPad = 1e-36f;
+        auto row_key = [&](int i) {
+            if (PKM) return f2ord(R[i]);
+            float n2 = kPad;
+            for (int be = 0; be < r; ++be) n2 = fmaf(R[be * Rp + i], R[be * Rp + i], n2);
+            return f2ord(n2);
+        };
+        auto my_rows = [&](auto f) {
+            for (int i = threadIdx.x; i < nr; i += kThreads) f(row_key(i));
+        };
+        uint32_t sm = 0u;
+        for (int j = threadIdx.x; j < K; j += kThreads) {
+            float n2 = kPad;
+            if (!PKM)
+                for (int be = 0; be < r; ++be) n2 = fmaf(S[be * Sp + j], S[be * Sp + j], n2);
+            sm = max(sm, f2ord(PKM ? S[j] : n2));
+        }
+        sm = __reduce_max_sync(kFull, sm);
+        if (lane == 0) atomicMax(&sh.smax, sm);
+        const uint32_t long_row = block_bound(kSeedRows, 16, sh.hist + 32, my_rows);
+        // the seeds: the first kSeedMax rows that reach it
+        float *seed = reinterpret_cast<float *>(stage);   // [r][kSeedMax]
+        int got = 0;
+        for (int i = threadIdx.x; i < nr; i += kThreads) got += row_key(i) >= long_row;
+        int seeds;
+        int at = block_scan(got, sh, &seeds);
+        for (int i = threadIdx.x; i < nr; i += kThreads)
+            if (row_key(i) >= long_row) {
+                if (at < kSeedMax)
+                    for (int be = 0; be < r; ++be) seed[be * kSeedMax + at] = R[be * Rp + i];
+                ++at;
             }
-        }
-        // 3. tau: the largest value with zero low bits that m group maxima
-        // reach (the leading kBoundBits of the key, from the top)
+        seeds = min(seeds, kSeedMax);
+        __syncthreads();
+        pad_rows(seed, kSeedMax, seeds);
+        const PassShape ps(seeds, K);
         uint32_t gk[kParts];
+        group_maxima<RP, PKM>(seed, kSeedMax, S, Sp, r, K, ps, gk);
+        const uint32_t tau0 = block_bound(m, kBoundBits, sh.hist + 64, [&](auto f) {
 #pragma unroll
-        for (int q = 0; q < kParts; ++q)
-            gk[q] = mine * (q + 1) / kParts > mine * q / kParts && kCols * cg < K ? f2ord(gm[q])
-                                                                                  : 0u;
-        uint32_t tau = 0u;
-#pragma unroll 1
-        for (int st = 0; st < kBoundBits; ++st) {
-            const uint32_t c = tau | (0x80000000u >> st);
-            int n = 0;
-#pragma unroll
-            for (int q = 0; q < kParts; ++q) n += gk[q] >= c;
-            n = __reduce_add_sync(kFull, n);
-            if (lane == 0 && n) atomicAdd(&sh.hist[st], n);
+            for (int q = 0; q < kParts; ++q) f(gk[q]);
+        });
+        const float t0 = ord2f(tau0), smax = ord2f(sh.smax);
+        // (tau0 = 0: fewer than m groups.)  The scores' rounding, at most a few
+        // ulps of |R| |S|, is far inside the margin 2^-12.
+        if (tau0 != 0u && (PKM || (t0 > 1e-12f && t0 < 1e18f))) {
+            auto keep = [&](int i) {
+                const uint32_t key = row_key(i);
+                if (PKM) return f2ord(ord2f(key) + smax) >= tau0;
+                return !(ord2f(key) * smax * (1.f + 1.f / 4096.f) < t0 * t0);
+            };
+            const int per_t = (nr + kThreads - 1) / kThreads;
+            const int lo = min(nr, (int)threadIdx.x * per_t), hi = min(nr, lo + per_t);
+            int mine = 0, kept;
+            for (int i = lo; i < hi; ++i) mine += keep(i);
+            int to = block_scan(mine, sh, &kept);
+            uint16_t *rows = reinterpret_cast<uint16_t *>(stage + 4 * kSeedMax * r);
+            for (int i = lo; i < hi; ++i)
+                if (keep(i)) rows[to++] = (uint16_t)i;
             __syncthreads();
-            if (sh.hist[st] >= m) tau = c;
+            // rows[i] >= i: whole batches move down without overwriting a later one
+            for (int base = 0; base < kept; base += kThreads) {
+                const int i = base + threadIdx.x;
+                float v[RP];
+#pragma unroll
+                for (int be = 0; be < RP; ++be)
+                    if (i < kept && be < r) v[be] = R[be * Rp + rows[i]];
+                __syncthreads();
+#pragma unroll
+                for (int be = 0; be < RP; ++be)
+                    if (i < kept && be < r) R[be * Rp + i] = v[be];
+                __syncthreads();
+            }
+            map = rows;
+            nr = kept;   // at least one: the rows that reach tau0
+            pad_rows(R, Rp, nr);
         }
-        // the groups that reach tau, a warp each: the pairs >= tau to the
+    }
+    const Grid gd{R, S, Rp, Sp, r, d.pkm};
+    if (!general) {
+        // 3. group maxima, and tau
+        const PassShape ps(nr, K);
+        uint32_t gk[kParts];
+        group_maxima<RP, PKM>(R, Rp, S, Sp, r, K, ps, gk);
+        const uint32_t tau = block_bound(m, kBoundBits, sh.hist, [&](auto f) {
+#pragma unroll
+            for (int q = 0; q < kParts; ++q) f(gk[q]);
+        });
+        // 4. the groups that reach tau, a warp each: the pairs >= tau to the
         // list (tau = 0, fewer than m groups: every pair)
 #pragma unroll
         for (int q = 0; q < kParts; ++q) {
             unsigned todo = __ballot_sync(kFull, gk[q] != 0u && gk[q] >= tau);
-            const int lo = mine * q / kParts, hi = mine * (q + 1) / kParts;
+            const int lo = ps.lo(q), hi = ps.lo(q + 1);
             while (todo) {
                 const int src = __ffs(todo) - 1;
                 todo &= todo - 1u;
                 const int glo = __shfl_sync(kFull, lo, src), ghi = __shfl_sync(kFull, hi, src);
-                const int grs = __shfl_sync(kFull, rs, src), gcg = __shfl_sync(kFull, cg, src);
+                const int grs = __shfl_sync(kFull, ps.rs, src);
+                const int gcg = __shfl_sync(kFull, ps.cg, src);
                 // an overflow is certain: stop early
                 if (__any_sync(kFull, *(volatile int *)&sh.count > list_n)) break;
                 for (int e = lane; e < 4 * (ghi - glo); e += 32) {
-                    const int i = 4 * (grs + (glo + (e >> 2)) * rs_n) + (e & 3);
+                    const int i = 4 * (grs + (glo + (e >> 2)) * ps.rs_n) + (e & 3);
                     if (i >= nr) continue;
+                    const uint32_t row = (uint32_t)(i0 + (map ? (int)map[i] : i)) * (uint32_t)K;
                     for (int j0 = kCols * gcg; j0 < K; j0 += kCols * kThreads)
                         for (int j = j0; j < min(j0 + kCols, K); ++j) {
                             const uint32_t key = f2ord(gd.score(i, j));
                             if (key >= tau) {
-                                const uint32_t v = (uint32_t)(i0 + i) * (uint32_t)K + (uint32_t)j;
                                 const int at = atomicAdd(&sh.count, 1);
-                                if (at < list_n) list[at] = comp_of(key, v);
+                                if (at < list_n) list[at] = comp_of(key, row + (uint32_t)j);
                             }
                         }
                 }
@@ -573,11 +843,11 @@ __global__ void __launch_bounds__(kThreads, 1)
         general = sh.count > list_n || sh.count < m;   // (fewer: never expected)
         __syncthreads();
     }
-    if (general) radix_top_m(gd, list, i0, nr, K, m, sh);
+    if (general) radix_top_m(gd, list, map, i0, nr, K, m, sh);
     const int n = min(sh.count, list_n);
     if (sh.count < m && threadIdx.x == 0) atomicOr(p.err, kErrInternal);   // never expected
 
-    // 4. ranks by (key desc, v asc): the number of composites above each
+    // 5. ranks by (key desc, v asc): the number of composites above each
     const int64_t base = (int64_t)pair * m;
     u64 *part = reinterpret_cast<u64 *>(p.akey) + ((int64_t)pair * shares + share) * m;
     for (int e = threadIdx.x; e < n; e += kThreads) {
@@ -649,15 +919,21 @@ cudaError_t configure_exact(const Dims &d) {
 cudaError_t launch_exact(const Dims &d, const Ptrs &p, int64_t *idx_out, float *w_out,
                          int *launches, cudaStream_t st) {
     const int shares = row_shares(d), rows = (d.K + shares - 1) / shares;
-    const int list = list_len(d, rows);
-    const size_t smem = exact_smem(d, rows, list);
+    // a stage where it fits beside a list of kMaxM, and the key rows allow
+    // 16-byte reads (dk % 32 == 0 makes their length do)
+    const size_t stage = stage_bytes_of(d, rows);
+    const int staged = d.dk % 32 == 0 && rows <= 65536 &&
+                       (((uintptr_t)p.k_row | (uintptr_t)p.k_col) & 15) == 0 &&
+                       exact_smem(d, rows, kMaxM) + stage + kStatic <= kSmemPerCta;
+    const int list = list_len(d, rows, staged ? stage : 0);
+    const size_t smem = exact_smem(d, rows, list) + (staged ? stage : 0);
     const int grid = d.B * d.H * shares;
     cudaError_t e = by_rank(d, [&](auto rp, auto pkm) {
         return d.dtype == ULTRAMEM_BF16
                    ? launch_kernel(d.pdl, exact_kernel<__nv_bfloat16, rp(), pkm()>, grid,
-                                   kThreads, smem, st, d, p, shares, list, idx_out, w_out)
+                                   kThreads, smem, st, d, p, shares, list, staged, idx_out, w_out)
                    : launch_kernel(d.pdl, exact_kernel<float, rp(), pkm()>, grid, kThreads, smem,
-                                   st, d, p, shares, list, idx_out, w_out);
+                                   st, d, p, shares, list, staged, idx_out, w_out);
     });
     *launches = shares > 1 ? 2 : 1;
     if (e == cudaSuccess && shares > 1)

@@ -26,6 +26,11 @@ CASES = [
     (dict(n=100, topk=32, topm=64, heads=1), 1),                   # 3 shares of rows
     (dict(n=150, rank=1, score_mode=1, d_k=64), 3),                # product keys
     (dict(n=150, rank=1, d_k=64, dtype=0), 3),
+    # 512 rows and more: rows that cannot hold a winner are dropped
+    (dict(n=300, d_k=128, heads=4), 40),                           # 16-byte stages, two a chunk
+    (dict(n=300, d_k=64, rank=1, score_mode=1, heads=4), 40),
+    (dict(n=300, d_k=64, dtype=0, heads=4, topk=32, topm=500), 40),
+    (dict(n=260, d_k=256, rank=4, heads=4), 40),
 ]
 
 
@@ -37,8 +42,9 @@ def test_exact_topm_layouts(case, gpu_lib):
     g_idx, g_w = layer.retrieve_exact(x)
     torch.cuda.synchronize()
     assert layer.check() == 0
-    o_idx, o_w = oracle.exact_topm(cfg, t, B)
-    _compare_exact(cfg, t, range(B), g_idx.cpu().numpy(), g_w.cpu().numpy(), o_idx, o_w)
+    tokens = np.unique(np.linspace(0, B - 1, min(B, 4)).astype(int))
+    o_idx, o_w = oracle.exact_topm(cfg, t, B, tokens=tokens)
+    _compare_exact(cfg, t, tokens, g_idx.cpu().numpy(), g_w.cpu().numpy(), o_idx, o_w)
     layer.close()
 
 
@@ -54,6 +60,22 @@ def test_ties_beyond_the_list(B, gpu_lib):
     g_idx, _ = layer.retrieve_exact(x)
     assert layer.check() == 0
     assert torch.equal(g_idx.cpu(), torch.arange(40).expand(B, cfg["heads"], 40))
+    layer.close()
+
+
+def test_equal_row_lengths_keep_every_row(gpu_lib):
+    """Keys of +-1/8 entries: every R has nearly the same length, so no row can
+    be dropped, and many scores tie."""
+    cfg = workloads.small_config(dtype=1, n=300, d_k=64, heads=4, topm=20)
+    w = workloads.make_weights(cfg, device="cuda")
+    for name in ("k_row", "k_col"):
+        w[name] = (w[name].float().sign() / 8).bfloat16()
+    layer, w, x, t = _layer(cfg, 40, w)
+    g_idx, g_w = layer.retrieve_exact(x)
+    assert layer.check() == 0
+    sample = np.array([0, 39])
+    o_idx, o_w = oracle.exact_topm(cfg, t, 40, tokens=sample)
+    _compare_exact(cfg, t, sample, g_idx.cpu().numpy(), g_w.cpu().numpy(), o_idx, o_w)
     layer.close()
 
 
