@@ -1685,10 +1685,11 @@ __device__ __forceinline__ int paired_q(int c, int lg) {
 // survivor's vector as soon as it has used one, so that NV loads a lane stay
 // in flight.  The scores go to srow [2 kWMaxK][RM] (scol is its second
 // half), zeros past the rank.
-template <int RM, int NV, int CH>
-__device__ __forceinline__ void warp_survivors(const Dims &d, const Ptrs &p, int h, int lg,
+template <int RM, int NV, int lg, int CH>
+__device__ __forceinline__ void warp_survivors(const Dims &d, const Ptrs &p, int h,
                                                const WarpSel &W) {
-    const int lane = threadIdx.x & 31, G = 1 << lg, sub = lane & (G - 1), per = 32 >> lg;
+    constexpr int G = 1 << lg, per = 32 >> lg;
+    const int lane = threadIdx.x & 31, sub = lane & (G - 1);
     const int n = 2 * d.k;
     int sv = lane >> lg;
     const uint4 *row = warp_row(d, p, h, sv, W.sel[0]) + sub;
@@ -1797,7 +1798,8 @@ __device__ __forceinline__ bool select_warp(const Dims &d, const Ptrs &p, int bh
     const int lg = survivor_lanes_log2(k);
     int nv = D >> (3 + lg);
     if (nv << (3 + lg) != D || d.r != CH || nv % CH || (nv & 1)) nv = 0;
-    const bool paired = nv == 8 || nv == 4 || (nv == 2 && CH <= 2);
+    const bool paired = (nv == 8 && lg == 1) || (nv == 4 && (lg == 1 || lg == 2)) ||
+                        (nv == 2 && CH <= 2 && (lg == 2 || lg == 3));
     // the row and column query of this (token, head)
     const int HD = d.H * D;
     for (int e = 4 * lane; e < 2 * D; e += 128) {
@@ -1841,9 +1843,13 @@ __device__ __forceinline__ bool select_warp(const Dims &d, const Ptrs &p, int bh
     }
     // the survivors' chunk scores (Eq. 4)
     const float *core = p.core + (int64_t)h * d.r * d.r;
-    if (paired && nv == 8) warp_survivors<RM, 8, CH>(d, p, h, lg, W);
-    else if (paired && nv == 4) warp_survivors<RM, 4, CH>(d, p, h, lg, W);
-    else if (paired) warp_survivors<RM, 2, (CH <= 2 ? CH : 1)>(d, p, h, lg, W);   // RM = 2
+    // (NV, lg) at compile time, so that the loads' offsets are immediates
+    if (paired && nv == 8) warp_survivors<RM, 8, 1, CH>(d, p, h, W);
+    else if (paired && nv == 4 && lg == 2) warp_survivors<RM, 4, 2, CH>(d, p, h, W);
+    else if (paired && nv == 4 && lg == 1) warp_survivors<RM, 4, 1, CH>(d, p, h, W);
+    else if (paired)   // 8 or 4 lanes, RM = 2
+        lg == 3 ? warp_survivors<RM, 2, 3, (CH <= 2 ? CH : 1)>(d, p, h, W)
+                : warp_survivors<RM, 2, 2, (CH <= 2 ? CH : 1)>(d, p, h, W);
     else warp_survivors_any<RM>(d, p, h, lg, W);
     __syncwarp();
     if (!warp_fold_rows<RM>(d, core, W)) return false;
