@@ -574,6 +574,8 @@ ultramem_status run(ultramem_layer *L, const Dims &d, Ptrs p, cudaStream_t st, R
     return s;
 }
 
+constexpr int kLongBackward = 512;   // tokens, see ultramem_lookup_reduce_backward
+
 // S7-S9 on given slots (p.idx_in, p.w_in): the lookup-reduce.  With slot_pos
 // the rows were looked up elsewhere (ultramem_shard_pool): slot s reads row
 // slot_pos[s] of p.values.
@@ -999,7 +1001,41 @@ ultramem_status ultramem_lookup_reduce_backward(ultramem_layer *L, const int64_t
     cudaError_t e;
     cudaGetLastError();
     int n = 0;
-    if (dw_proj && d.has_proj) {
+    // Long batches on the tensor cores (whole 16-byte rows): the gather works
+    // the slots out, dW_p reads g and the pooled rows as they are (tokens along
+    // the rows of both), and the kernels are programmatic dependents of one
+    // another (g and the slots were complete before the first).  Measured on
+    // GB300, decode_1m with 2048 tokens: 301 -> 256 us a call (137 of it zeroing
+    // dV); below 512 tokens the separate slots, transposes and plain launches
+    // stay.
+    bool chained = false;
+    if (dw_proj && d.has_proj && L->tc && L->dacc_tc && B >= kLongBackward &&
+        L->cfg.d_out % 8 == 0) {
+        const int kd = d.E * d.d_v;
+        CUtensorMap am, gm;
+        Ptrs pg = p;
+        pg.acc_bf = L->ws.acc_bf;   // [B][2][E D_v]
+        pg.acc_terms = 2;
+        bool gathered = false;
+        if (um::tc_encode(&am, L->ws.acc_bf, 2ull * kd, (uint64_t)B, 1, 64, 2) &&
+            um::tc_encode(&gm, g, (uint64_t)L->cfg.d_out, (uint64_t)B, 1, 64, 2)) {
+            if ((e = um::launch_gather_addresses(d, pg, &gathered, st)) != cudaSuccess)
+                return from_cuda(e);
+            n = 1;
+            if (!gathered) {
+                if ((e = um::launch_slots_from_addresses(d, p, st)) != cudaSuccess ||
+                    (e = um::launch_gather(d, pg, st)) != cudaSuccess)
+                    return from_cuda(e);
+                n = 2;
+            }
+            d.pdl = 1;
+            if ((e = um::launch_dw_mn(d, gm, am, dw_proj, L->ws.err, st)) != cudaSuccess)
+                return from_cuda(e);
+            ++n;
+            chained = true;
+        }
+    }
+    if (dw_proj && d.has_proj && !chained) {
         // dW_p needs the forward's pooled rows: the forward's slots and gather
         if ((e = um::launch_slots_from_addresses(d, p, st)) != cudaSuccess) return from_cuda(e);
         const int kd = d.E * d.d_v;
@@ -1045,7 +1081,7 @@ ultramem_status ultramem_lookup_reduce_backward(ultramem_layer *L, const int64_t
             um::TcMaps mp = L->maps;
             CUtensorMap gm;
             if (um::tc_encode(&gm, g, (uint64_t)d.d_out, (uint64_t)B, 1,
-                              (uint32_t)um::tc_n_tile(B, 1), 2)) {
+                              (uint32_t)um::dacc_token_box(d), 2)) {
                 if ((e = um::launch_dacc_tc(d, mp.w_p, gm, L->ws.dacc, L->ws.err, st)) !=
                     cudaSuccess)
                     return from_cuda(e);

@@ -147,6 +147,8 @@ __global__ void __launch_bounds__(kThreads) rows_kernel(Dims d, Ptrs p, const vo
     const int Dv = d.d_v, EDv = d.E * Dv, nc = d.nc, hm = d.H * d.m;
     const int lane = threadIdx.x & 31;
     const int64_t slot = (int64_t)blockIdx.x * kWarps + (threadIdx.x >> 5);
+    pdl_wait();
+    pdl_trigger();
     if (slot >= (int64_t)d.B * hm) return;   // warp-uniform
     const int64_t b = slot / hm;
     const bool active = lane * EPV < Dv;
@@ -238,11 +240,11 @@ cudaError_t launch_backward_rows(const Dims &d, const Ptrs &p, const void *g, fl
     const void *src = d.has_proj ? static_cast<const void *>(dacc) : g;
     const int64_t slots = (int64_t)d.B * d.H * d.m;
     const unsigned blocks = (unsigned)((slots + kWarps - 1) / kWarps);
-    if (bf)
-        rows_kernel<__nv_bfloat16><<<blocks, kThreads, 0, st>>>(d, p, src, dV, dw);
-    else
-        rows_kernel<float><<<blocks, kThreads, 0, st>>>(d, p, src, dV, dw);
-    return cudaGetLastError();
+    // a dependent of the dacc contraction when that is the kernel before it
+    const bool pdl = d.pdl && d.has_proj && dacc_ready;
+    return bf ? launch_kernel(pdl, rows_kernel<__nv_bfloat16>, blocks, kThreads, 0, st, d, p, src,
+                              dV, dw)
+              : launch_kernel(pdl, rows_kernel<float>, blocks, kThreads, 0, st, d, p, src, dV, dw);
 }
 
 // dW_p from the forward's pooled rows acc (fp32 [B][E D_v]) and g.

@@ -186,6 +186,21 @@ __device__ __forceinline__ uint64_t desc_k_sw128(uint32_t saddr) {
     return d;
 }
 
+// Shared-memory matrix descriptor of an MN-major tile written by TMA with the
+// 128-byte swizzle: boxes of 64 K rows x 128 bytes (64 elements along M or
+// N), 8-row groups of K 1024 bytes apart, the next 64 elements a box (8192
+// bytes) on.
+__device__ __forceinline__ uint64_t desc_mn_sw128(uint32_t saddr) {
+    uint64_t d = 0;
+    d |= (uint64_t)((saddr & 0x3FFFFu) >> 4);   // start address >> 4, bits [0,14)
+    d |= (uint64_t)(8192 >> 4) << 16;           // leading byte offset: the next 64 along M/N
+    d |= (uint64_t)(1024 >> 4) << 32;           // stride byte offset: the next 8 along K
+    d |= (uint64_t)1 << 46;                     // descriptor version for tcgen05
+    d |= (uint64_t)2 << 61;                     // 128-byte swizzle
+    return d;
+}
+constexpr uint32_t kIdescMnMajor = (1u << 15) | (1u << 16);   // A and B are MN-major
+
 // Instruction descriptor of kind::f16 with bf16 A and B, fp32 D, both K-major.
 __host__ __device__ constexpr uint32_t idesc_bf16_f32(int M, int N) {
     return (1u << 4)                       // D format: f32

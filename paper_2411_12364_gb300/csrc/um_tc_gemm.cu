@@ -107,6 +107,18 @@ template <class Op> struct ARows<Op, std::void_t<decltype(Op::kARows)>> {
     static constexpr int value = Op::kARows;
 };
 
+// An op with kMnMajor = true reads operands whose rows run along K (the
+// contraction sums over the rows of both): boxes of 64 K rows x 64 columns,
+// MN-major tiles of the MMA.  No transposed copies.  (One-CTA-per-tile
+// kernel only; n_tile a multiple of 64.)
+template <class Op, class = void> struct MnMajor {
+    static constexpr bool value = false;
+};
+template <class Op> struct MnMajor<Op, std::void_t<decltype(Op::kMnMajor)>> {
+    static constexpr bool value = Op::kMnMajor;
+};
+constexpr uint32_t kMnBoxBytes = 64 * 128;   // 64 K rows of 64 bf16
+
 // An op with kGroupEpilogue = true (the candidate-list passes: swapped)
 // reduces each group of 16 accumulator columns to one 32-bit value (group)
 // and stores a thread's consecutive groups at once (store_groups): each
@@ -212,6 +224,12 @@ __global__ void __launch_bounds__(kThreads, 1)
         uint8_t *sa = ring + (size_t)s * stage_bytes;
         mbar_arrive_expect_tx(&full[s], stage_bytes);
         const int kx = (t.kb0 + it) * kBlockK;
+        if constexpr (MnMajor<Op>::value) {
+#pragma unroll
+            for (int i = 0; i < kTileM / 64; ++i)
+                tma_load_2d(sa + i * kMnBoxBytes, mapA, &full[s], t.m0 + 64 * i, kx);
+            return;
+        }
 #pragma unroll
         for (int ab = 0; ab < kA / kTileM; ++ab) {
             uint8_t *sab = sa + ab * kTileABytes;
@@ -226,6 +244,12 @@ __global__ void __launch_bounds__(kThreads, 1)
 #pragma unroll
         for (int j = 0; j < NSPLIT; ++j) {
             uint8_t *sb = sa + a_bytes + j * b_bytes;
+            if constexpr (MnMajor<Op>::value) {
+                for (int i = 0; i < n_tile / 64; ++i)
+                    tma_load_2d(sb + i * kMnBoxBytes, &mapB, &full[s],
+                                j * op.b_split_stride + t.n0 + 64 * i, kx);
+                continue;
+            }
             const int bx = j * op.b_split_stride + kx;
             if (t.b_z >= 0) tma_load_3d(sb, &mapB, &full[s], bx, t.n0, t.b_z);
             else tma_load_2d(sb, &mapB, &full[s], bx, t.n0);
@@ -271,7 +295,11 @@ __global__ void __launch_bounds__(kThreads, 1)
         // MMA issuer.  Descriptors are built once per stage and advanced by
         // 32 bytes (2 in the >>4 address field) per 16-wide K step; the
         // accumulator of each step follows its rank chunk without division.
-        const uint32_t idesc = kSwap ? idesc_bf16_f32(n_tile, kA) : idesc_bf16_f32(kTileM, n_tile);
+        constexpr bool kMn = MnMajor<Op>::value;
+        const uint32_t idesc = (kSwap ? idesc_bf16_f32(n_tile, kA) : idesc_bf16_f32(kTileM, n_tile)) |
+                               (kMn ? kIdescMnMajor : 0u);
+        // the descriptors' step per 16 K: 32 bytes of a row, or 16 rows
+        constexpr int kStep = kMn ? 16 * 128 >> 4 : 32 >> 4;
         uint32_t started = 0;
         int acc = (t.kb0 * kBlockK) / op.acc_chunk;
         int next_chunk = (acc + 1) * op.acc_chunk;   // K index where acc advances
@@ -283,10 +311,11 @@ __global__ void __launch_bounds__(kThreads, 1)
             }
             tc_fence_after();
             const uint32_t sa = smem_u32(ring + (size_t)s * stage_bytes);
-            const uint64_t ad0 = desc_k_sw128(sa);
+            const uint64_t ad0 = kMn ? desc_mn_sw128(sa) : desc_k_sw128(sa);
             uint64_t bd0[NSPLIT];
 #pragma unroll
-            for (int j = 0; j < NSPLIT; ++j) bd0[j] = desc_k_sw128(sa + a_bytes + j * b_bytes);
+            for (int j = 0; j < NSPLIT; ++j) bd0[j] = kMn ? desc_mn_sw128(sa + a_bytes + j * b_bytes)
+                             : desc_k_sw128(sa + a_bytes + j * b_bytes);
 #pragma unroll
             for (int k16 = 0; k16 < kBlockK / 16; ++k16) {
                 const int kg = (t.kb0 + it) * kBlockK + k16 * 16;
@@ -299,9 +328,9 @@ __global__ void __launch_bounds__(kThreads, 1)
 #pragma unroll
                 for (int j = 0; j < NSPLIT; ++j) {
                     if constexpr (kSwap)
-                        mma_bf16(dt, bd0[j] + 2 * k16, ad0 + 2 * k16, idesc, started & acc_bit);
+                        mma_bf16(dt, bd0[j] + kStep * k16, ad0 + kStep * k16, idesc, started & acc_bit);
                     else
-                        mma_bf16(dt, ad0 + 2 * k16, bd0[j] + 2 * k16, idesc, started & acc_bit);
+                        mma_bf16(dt, ad0 + kStep * k16, bd0[j] + kStep * k16, idesc, started & acc_bit);
                     started |= acc_bit;
                 }
             }
@@ -1073,6 +1102,13 @@ struct DwOp {
     }
 };
 
+// The same from the operands as they are: A = the gradient rows g [B][D'_v],
+// B = the pooled rows' terms acc [B][2][E D_v] (the lo term at column offset
+// E D_v), both with the tokens along the rows (kMnMajor).
+struct DwMnOp : DwOp {
+    static constexpr bool kMnMajor = true;
+};
+
 // dst[c][r] = src[r][c] for a rows x cols bf16 matrix (32 x 32 tiles), with
 // row strides ld_src (>= cols) and ld_dst (>= rows) in elements
 __global__ void transpose_kernel(const __nv_bfloat16 *__restrict__ src,
@@ -1225,6 +1261,9 @@ cudaError_t configure_tc() {
     if (e == cudaSuccess) e = allow_smem<3, ProjRowsOp<256>>();
     if (e == cudaSuccess) e = allow_smem<1, DaccOp>();
     if (e == cudaSuccess) e = allow_smem<2, DwOp>();
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(tc_gemm_kernel<2, DwMnOp>,
+                                 cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBudget);
     return e;
 }
 
@@ -1245,11 +1284,45 @@ cudaError_t launch_dw_tc(const Dims &d, const CUtensorMap &g_t, const CUtensorMa
     return launch_gemm<2>(grid, g_t, g_t, acc_t2, op, op.kb_total, false, st);
 }
 
+cudaError_t launch_dw_mn(const Dims &d, const CUtensorMap &g, const CUtensorMap &acc2, float *dW,
+                         int *err, cudaStream_t st) {
+    DwMnOp op;
+    op.stamp = nullptr;
+    op.M = d.d_out;
+    op.N = d.E * d.d_v;
+    // columns a tile: as many (64 to 256) as still leave a CTA for most SMs.
+    // With 256 decode_1m's 1024 x 1024 gradient ran on 32 CTAs: 27 us over 2048
+    // tokens, 20 with 64 (L2 reads of the operands).
+    const int m_tiles = (op.M + kTileM - 1) / kTileM;
+    op.n_tile = 256;
+    while (op.n_tile > 64 &&
+           (op.n_tile >= 2 * op.N ||
+            4 * m_tiles * ((op.N + op.n_tile - 1) / op.n_tile) < 3 * sm_count()))
+        op.n_tile /= 2;
+    op.n_acc = 1;
+    op.acc_chunk = 1 << 30;
+    op.b_split_stride = op.N;   // the lo term follows the hi term in a row
+    op.err = err;
+    op.kb_total = (d.B + kBlockK - 1) / kBlockK;
+    op.out = dW;
+    dim3 grid(m_tiles, (op.N + op.n_tile - 1) / op.n_tile, 1);
+    op.stages = stages_for(2, op.n_tile, op.kb_total);
+    const size_t smem = 1024 + (size_t)op.stages * stage_bytes_of(2, op.n_tile);
+    return launch_kernel(d.pdl, 1u, tc_gemm_kernel<2, DwMnOp>, grid, kThreads, smem, st, g, g,
+                         acc2, op, 0);
+}
+
+// tokens a tile of the dacc contraction: 128 where 256 would leave SMs idle
+int dacc_token_box(const Dims &d) {
+    const int nt = tc_n_tile(d.B, 1);
+    const int64_t tiles = (int64_t)((d.E * d.d_v + kTileM - 1) / kTileM) * ((d.B + nt - 1) / nt);
+    return nt > 128 && tiles < sm_count() ? 128 : nt;
+}
 cudaError_t launch_dacc_tc(const Dims &d, const CUtensorMap &w_p, const CUtensorMap &g,
                            float *dacc, int *err, cudaStream_t st) {
     DaccOp op;
     op.stamp = nullptr;
-    op.n_tile = tc_n_tile(d.B, 1);
+    op.n_tile = dacc_token_box(d);
     op.n_acc = 1;
     op.acc_chunk = 1 << 30;
     op.b_split_stride = 0;
@@ -1259,7 +1332,7 @@ cudaError_t launch_dacc_tc(const Dims &d, const CUtensorMap &w_p, const CUtensor
     op.kb_total = (d.d_out + kBlockK - 1) / kBlockK;
     op.out = dacc;
     dim3 grid((op.M + kTileM - 1) / kTileM, (d.B + op.n_tile - 1) / op.n_tile, 1);
-    return launch_gemm<1>(grid, w_p, w_p, g, op, op.kb_total, false, st);
+    return launch_gemm<1>(grid, w_p, w_p, g, op, op.kb_total, d.pdl, st);
 }
 
 // x_splits: the B operand is the convolved input as three bf16 terms (map
