@@ -72,6 +72,102 @@ __global__ void __launch_bounds__(kThreads) conv_kernel(Dims d, Ptrs p, int spli
     stamp_end(p.stamp);
 }
 
+// The same for bf16 rows of whole 16-byte vectors (aligned): a thread takes 8
+// channels of TPT tokens in a row, so that inputs and terms move 16 bytes at a
+// time and the taps are read once for all of them.  Sums in the same order.
+// Measured on GB300 (4 taps, 1024 channels): 2000 tokens 17.2 -> 8.4 us.
+__device__ __forceinline__ void bf16x8(uint4 v, float (&f)[8]) {
+    const uint32_t u[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        f[2 * q] = __uint_as_float(u[q] << 16);
+        f[2 * q + 1] = __uint_as_float(u[q] & 0xffff0000u);
+    }
+}
+// the 8 inputs at channel c, j tokens before token b (see input_back)
+__device__ __forceinline__ uint4 input_back8(const Dims &d, const Ptrs &p, int b, int j, int c) {
+    const int s = b / d.seq_len, pos = b - s * d.seq_len - j;
+    const __nv_bfloat16 *src;
+    if (pos >= 0) {
+        src = static_cast<const __nv_bfloat16 *>(p.x) + (int64_t)(b - j) * d.d_in;
+    } else {
+        if (!p.state_in) return make_uint4(0, 0, 0, 0);
+        const int kk = d.conv_k - 1;
+        src = static_cast<const __nv_bfloat16 *>(p.state_in) +
+              ((int64_t)s * kk + kk + pos) * d.d_in;
+    }
+    return *reinterpret_cast<const uint4 *>(src + c);
+}
+template <int TPT>
+__global__ void __launch_bounds__(kThreads) conv8_kernel(Dims d, Ptrs p, int splits,
+                                                         int state_rows) {
+    pdl_wait();
+    stamp_begin(p.stamp);
+    pdl_trigger();
+    const int nv = d.d_in >> 3, groups = (d.B + TPT - 1) / TPT;
+    const int64_t e = (int64_t)blockIdx.x * kThreads + threadIdx.x;
+    const int unit = (int)(e / nv), c = 8 * (int)(e - (int64_t)unit * nv);
+    if (unit < groups) {
+        float acc[TPT][8];
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            const float b0 = p.conv_b ? p.conv_b[c + k] : 0.f;
+#pragma unroll
+            for (int t = 0; t < TPT; ++t) acc[t][k] = b0;
+        }
+        for (int j = 0; j < d.conv_k; ++j) {
+            const float4 *wp = reinterpret_cast<const float4 *>(p.conv_w + (int64_t)j * d.d_in + c);
+            const float4 w0 = wp[0], w1 = wp[1];
+            const float w[8] = {w0.x, w0.y, w0.z, w0.w, w1.x, w1.y, w1.z, w1.w};
+            uint4 x[TPT];
+#pragma unroll
+            for (int t = 0; t < TPT; ++t)
+                x[t] = input_back8(d, p, min(unit * TPT + t, d.B - 1), j, c);
+#pragma unroll
+            for (int t = 0; t < TPT; ++t) {
+                float f[8];
+                bf16x8(x[t], f);
+#pragma unroll
+                for (int k = 0; k < 8; ++k) acc[t][k] = fmaf(w[k], f[k], acc[t][k]);
+            }
+        }
+#pragma unroll
+        for (int t = 0; t < TPT; ++t) {
+            const int b = unit * TPT + t;
+            if (b >= d.B) break;
+            if (splits) {
+                __nv_bfloat16 *dst = static_cast<__nv_bfloat16 *>(p.xs) + (int64_t)b * 3 * d.d_in + c;
+#pragma unroll
+                for (int term = 0; term < 3; ++term) {
+                    uint32_t u[4];
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) {
+                        const __nv_bfloat162 h =
+                            __floats2bfloat162_rn(acc[t][2 * k], acc[t][2 * k + 1]);
+                        u[k] = *reinterpret_cast<const uint32_t *>(&h);
+                        acc[t][2 * k] -= __low2float(h);
+                        acc[t][2 * k + 1] -= __high2float(h);
+                    }
+                    *reinterpret_cast<uint4 *>(dst + term * d.d_in) =
+                        make_uint4(u[0], u[1], u[2], u[3]);
+                }
+            } else {
+                float4 *dst = reinterpret_cast<float4 *>(static_cast<float *>(p.xs) +
+                                                         (int64_t)b * d.d_in + c);
+                dst[0] = make_float4(acc[t][0], acc[t][1], acc[t][2], acc[t][3]);
+                dst[1] = make_float4(acc[t][4], acc[t][5], acc[t][6], acc[t][7]);
+            }
+        }
+    } else if (unit < groups + state_rows) {
+        // state row i of sequence s: input seq_len - kk + i of it (a copy)
+        const int kk = d.conv_k - 1, row = unit - groups, s = row / kk, i = row - s * kk;
+        __nv_bfloat16 *dst = static_cast<__nv_bfloat16 *>(p.state_out) + (int64_t)row * d.d_in + c;
+        *reinterpret_cast<uint4 *>(dst) =
+            input_back8(d, p, s * d.seq_len + d.seq_len - 1, kk - 1 - i, c);
+    }
+    stamp_end(p.stamp);
+}
+
 __device__ __forceinline__ float warp_sum(float v) {
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(kFull, v, off);
@@ -211,6 +307,19 @@ __global__ void __launch_bounds__(kThreads) key_ln_kernel(const T *keys, int64_t
 cudaError_t launch_query_conv(const Dims &d, const Ptrs &p, bool splits, cudaStream_t st) {
     const int seqs = d.B / d.seq_len;
     const int state_rows = p.state_out ? seqs * (d.conv_k - 1) : 0;
+    const uintptr_t at = (uintptr_t)p.x | (uintptr_t)p.conv_w | (uintptr_t)p.state_in |
+                         (uintptr_t)p.state_out;
+    if (d.dtype == ULTRAMEM_BF16 && d.d_in % 8 == 0 && (at & 15) == 0) {
+        const int nv = d.d_in / 8;
+        auto go = [&](auto kernel, int tpt) {
+            const int64_t units = (d.B + tpt - 1) / tpt + state_rows;
+            return launch_kernel(d.pdl, kernel, (unsigned)((units * nv + kThreads - 1) / kThreads),
+                                 kThreads, 0, st, d, p, splits ? 1 : 0, state_rows);
+        };
+        // four tokens a thread once that leaves a CTA for every SM
+        return (int64_t)d.B * nv >= 4ll * kThreads * device_sm_count() ? go(conv8_kernel<4>, 4)
+                                                                       : go(conv8_kernel<1>, 1);
+    }
     dim3 grid(d.B + state_rows, (d.d_in + kThreads - 1) / kThreads);
     if (d.dtype == ULTRAMEM_BF16)
         return launch_kernel(d.pdl, conv_kernel<__nv_bfloat16>, grid, kThreads, 0, st, d, p,
