@@ -1183,10 +1183,10 @@ __device__ __forceinline__ void select_block(const Dims &d, const Ptrs &p, int b
     };
     double gmax_d = 0.0;
     if constexpr (kExact) {
-        int i0, j0;
-        pair_of(fwin[0], i0, j0);
-        gmax_d = exact_g(i0, j0, sh.core);
         if (d.act == ULTRAMEM_ACT_SOFTMAX) {
+            int i0, j0;
+            pair_of(fwin[0], i0, j0);
+            gmax_d = exact_g(i0, j0, sh.core);
             if (threadIdx.x < 32) {
                 double z = 0.0;
                 for (int e = threadIdx.x; e < m; e += 32) {
