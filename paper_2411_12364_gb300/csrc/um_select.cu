@@ -1,4 +1,5 @@
-// um_select.cu -- S4..S7 for one (token, head) per CTA:
+// um_select.cu -- S4..S7 for one (token, head) per CTA (on long grids one per
+// warp, select_warp_kernel below, with the same results):
 //   top-k of each axis on the rank-1 score keys         (Eq. 8-9)
 //   exact chunk scores S_alpha of the 2k survivors      (Eq. 4)
 //   exact Tucker score g on the k*k survivor pairs      (Eq. 10; with product
@@ -12,7 +13,7 @@
 // scores of the k survivors of each axis are recomputed here from q and the
 // key rows.  Ties go to the smaller index.
 //
-// Top-k of n keys, in two stages.  Candidates: each thread keeps the two
+// Top-k of n keys in a CTA, in two stages.  Candidates: each thread keeps the two
 // largest of its share of the keys; each warp takes the j-th largest of its
 // lanes' 64 values (j = ceil(k / 8): j rounds of a warp max that removes one
 // instance) and tau is the smallest of the 8 warp values.  Every warp owns at
