@@ -183,56 +183,37 @@ size_t bucket_smem_bytes(const Dims &d, int warps) {
            sizeof(float) * (size_t)hm * d.nc;
 }
 
-// THREADS = 512 (2 CTAs per SM) for batches up to about two CTAs per SM,
-// where each token's latency matters; 256 (4 CTAs per SM) for longer
-// grids, where CTAs in their bucketing or reduction phase overlap others'
-// loads (measured: 6.5 TB/s over 2.15 GB at 16384 tokens, against 5.4 with
-// 512).
-// ADDR: the slots come as given addresses and weights (p.idx_in, p.w_in)
-// instead of the selection's sel_row / sel_p / sel_w, and each thread works
-// its slot out itself: the slots kernel before the gather, its launch and
-// the round trip of 12 bytes a slot through memory go.
-// VPL: 16-byte vectors of a row that a lane owns (2: fp32 rows of up to 256
-// values; half as many rows in flight).  fp32 rows' fp64 sums take twice the
-// registers, so half as many CTAs per SM.
-template <typename T, int THREADS, bool ADDR, int VPL = 1>
-__global__ void __launch_bounds__(THREADS, (sizeof(T) == 4 ? 512 : 1024) / THREADS)
-    gather_bucket_kernel(Dims d, Ptrs p) {
-    constexpr int kBThreads = THREADS, kBWarps = THREADS / 32, kRows = kUnroll / VPL;
-    extern __shared__ __align__(16) unsigned char gsm[];
-    __shared__ int wcnt[kBWarps][kBMaxE];   // per warp and block: count, then offset
-    __shared__ int tot[kBMaxE], start[kBMaxE];
-    constexpr int EPV = 16 / sizeof(T);
-    const int b = blockIdx.x, E = d.E, hm = d.H * d.m, Dv = d.d_v;
+// The bucketed gathers' slots: a stable counting sort of token b's slots by
+// block (slot order kept within a block) into row_s and w_s, block q's at
+// start[q] .. start[q] + tot[q].  ADDR: the slots come as given addresses and
+// weights (p.idx_in, p.w_in) instead of the selection's sel_row / sel_p /
+// sel_w, and each thread works its slot out itself: the slots kernel before
+// the gather, its launch and the round trip of 12 bytes a slot through memory
+// go.  Whole block; ends with a barrier.
+template <int THREADS, bool ADDR>
+__device__ __forceinline__ void bucket_slots(const Dims &d, const Ptrs &p, int64_t base, int hm,
+                                             int (*wcnt)[kBMaxE], int *tot, int *start,
+                                             int *row_s, float *w_s) {
+    constexpr int kBWarps = THREADS / 32;
+    const int E = d.E, nc = d.nc;
     const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
-    const int64_t base = (int64_t)b * hm;
-    // the warps' sums [kBWarps][D_v]: fp32, or (fp32 storage) s and c of Dot2
-    using R = typename std::conditional<std::is_same<T, float>::value, float2, float>::type;
-    R *red = reinterpret_cast<R *>(gsm);
-    int *row_s = reinterpret_cast<int *>(red + kBWarps * Dv);    // [hm] bucketed rows
-    float *w_s = reinterpret_cast<float *>(row_s + hm);          // [hm][nc] their weights
-    const int nc = d.nc;
-    pdl_wait();
-    stamp_begin(p.stamp);
-    pdl_trigger();
-
-    // stable counting sort of the slots by block (slot order kept within a block)
     int row = 0, blk = -1;
     float w[kMaxCores];   // the slot's weight, or its nc slice weights (MCS)
 #pragma unroll
     for (int ci = 0; ci < kMaxCores; ++ci) w[ci] = 0.f;
     if (t < hm) {
-        bool ok = true;   // an invalid address weighs 0
-        if constexpr (ADDR) {
-            ok = slot_of_address(d, p, p.idx_in[base + t], row, blk);
+        if constexpr (ADDR) {   // an invalid address weighs 0
+            const bool ok = slot_of_address(d, p, p.idx_in[base + t], row, blk);
+#pragma unroll
+            for (int ci = 0; ci < kMaxCores; ++ci)
+                if (ci < nc) w[ci] = ok ? p.w_in[(base + t) * nc + ci] : 0.f;
         } else {
             row = p.sel_row[base + t];
             blk = p.sel_p[base + t];
-        }
-        const float *ws = ADDR ? p.w_in : p.sel_w;
 #pragma unroll
-        for (int ci = 0; ci < kMaxCores; ++ci)
-            if (ci < nc) w[ci] = ok ? ws[(base + t) * nc + ci] : 0.f;
+            for (int ci = 0; ci < kMaxCores; ++ci)
+                if (ci < nc) w[ci] = p.sel_w[(base + t) * nc + ci];
+        }
         if (blk < 0 || blk >= E) blk = -1;   // not a slot of this layer: skipped
     }
     int rank = 0;
@@ -268,6 +249,105 @@ __global__ void __launch_bounds__(THREADS, (sizeof(T) == 4 ? 512 : 1024) / THREA
             if (ci < nc) w_s[pos * nc + ci] = w[ci];
     }
     __syncthreads();
+}
+
+// The bucketed gather of bf16 rows (a 16-byte vector a lane).
+// THREADS = 512 (2 CTAs per SM) for batches up to about two CTAs per SM,
+// where each token's latency matters; 256 (4 CTAs per SM) for longer
+// grids, where CTAs in their bucketing or reduction phase overlap others'
+// loads (measured: 6.5 TB/s over 2.15 GB at 16384 tokens, against 5.4 with
+// 512).  fp32 rows have a kernel of their own below: as one template with
+// theirs this one's code came out slower, 3.2 -> 3.7 us at decode_1m with 64
+// tokens, 4.6 -> 5.2 at mid_4m with 32.
+template <int THREADS, bool ADDR>
+__global__ void __launch_bounds__(THREADS, 1024 / THREADS) gather_bucket_kernel(Dims d, Ptrs p) {
+    using T = __nv_bfloat16;
+    constexpr int kBThreads = THREADS, kBWarps = THREADS / 32;
+    extern __shared__ __align__(16) unsigned char gsm[];
+    __shared__ int wcnt[kBWarps][kBMaxE];   // per warp and block: count, then offset
+    __shared__ int tot[kBMaxE], start[kBMaxE];
+    constexpr int EPV = 16 / sizeof(T);
+    const int b = blockIdx.x, E = d.E, hm = d.H * d.m, Dv = d.d_v;
+    const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
+    const int64_t base = (int64_t)b * hm;
+    float *red = reinterpret_cast<float *>(gsm);                 // [kBWarps][D_v]
+    int *row_s = reinterpret_cast<int *>(red + kBWarps * Dv);    // [hm] bucketed rows
+    float *w_s = reinterpret_cast<float *>(row_s + hm);          // [hm][nc] their weights
+    const int nc = d.nc;
+    pdl_wait();
+    stamp_begin(p.stamp);
+    pdl_trigger();
+    bucket_slots<THREADS, ADDR>(d, p, base, hm, wcnt, tot, start, row_s, w_s);
+
+    // warps [q*wpb, (q+1)*wpb) serve block q, each a contiguous share
+    const int wpb = kBWarps / E;
+    const int q = warp / wpb, sub = warp - q * wpb;
+    const bool active = lane * EPV < Dv;
+    const int wsel = nc == 1 || !active ? 0 : (lane * EPV) / (Dv / nc);   // this lane's slice
+    const T *V = static_cast<const T *>(p.values) + lane * EPV;
+    float acc[EPV];
+#pragma unroll
+    for (int c = 0; c < EPV; ++c) acc[c] = 0.f;
+    if (q < E) {
+        const int n = tot[q], per = (n + wpb - 1) / wpb;
+        const int lo = start[q] + min(n, sub * per), hi = start[q] + min(n, (sub + 1) * per);
+        for (int j0 = lo; j0 < hi; j0 += kUnroll) {
+            uint4 val[kUnroll];
+            float wu[kUnroll];
+#pragma unroll
+            for (int u = 0; u < kUnroll; ++u) {
+                const int j = j0 + u;
+                const bool ok = j < hi;
+                wu[u] = ok ? w_s[j * nc + wsel] : 0.f;
+                val[u] = (ok && active) ? ld_stream(V + (int64_t)row_s[j] * Dv)
+                                        : make_uint4(0, 0, 0, 0);
+            }
+#pragma unroll
+            for (int u = 0; u < kUnroll; ++u) {
+                float f[EPV];
+                unpack<T>(val[u], f);
+#pragma unroll
+                for (int c = 0; c < EPV; ++c) acc[c] = mul_add(wu[u], f[c], acc[c]);
+            }
+        }
+        if (active)
+#pragma unroll
+            for (int c = 0; c < EPV; ++c) red[warp * Dv + lane * EPV + c] = acc[c];
+    }
+    __syncthreads();
+    const int EDv = E * Dv;
+    for (int i = t; i < EDv; i += kBThreads) {
+        const int qq = i / Dv, c = i - qq * Dv;
+        float sum = 0.f;
+        for (int sb = 0; sb < wpb; ++sb) sum += red[(qq * wpb + sb) * Dv + c];
+        store_pooled<T>(d, p, b, i, sum);
+    }
+    stamp_end(p.stamp);
+}
+
+// The same for fp32 rows, with compensated sums (Dot2).  VPL: 16-byte vectors
+// of a row that a lane owns (2: rows of up to 256 values; half as many rows in
+// flight).  A sum and its error term take twice the registers of a plain sum,
+// so half as many CTAs per SM.
+template <int THREADS, int VPL>
+__global__ void __launch_bounds__(THREADS, 512 / THREADS) gather_bucket_exact(Dims d, Ptrs p) {
+    using T = float;
+    constexpr int kBThreads = THREADS, kBWarps = THREADS / 32, kRows = kUnroll / VPL;
+    extern __shared__ __align__(16) unsigned char gsm[];
+    __shared__ int wcnt[kBWarps][kBMaxE];   // per warp and block: count, then offset
+    __shared__ int tot[kBMaxE], start[kBMaxE];
+    constexpr int EPV = 16 / sizeof(T);
+    const int b = blockIdx.x, E = d.E, hm = d.H * d.m, Dv = d.d_v;
+    const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
+    const int64_t base = (int64_t)b * hm;
+    float2 *red = reinterpret_cast<float2 *>(gsm);   // the warps' s and c of Dot2 [kBWarps][D_v]
+    int *row_s = reinterpret_cast<int *>(red + kBWarps * Dv);    // [hm] bucketed rows
+    float *w_s = reinterpret_cast<float *>(row_s + hm);          // [hm][nc] their weights
+    const int nc = d.nc;
+    pdl_wait();
+    stamp_begin(p.stamp);
+    pdl_trigger();
+    bucket_slots<THREADS, false>(d, p, base, hm, wcnt, tot, start, row_s, w_s);
 
     // warps [q*wpb, (q+1)*wpb) serve block q, each a contiguous share
     const int wpb = kBWarps / E;
@@ -281,14 +361,7 @@ __global__ void __launch_bounds__(THREADS, (sizeof(T) == 4 ? 512 : 1024) / THREA
         wsel[x] = nc == 1 || !active[x] ? 0 : c0 / (Dv / nc);
     }
     const T *V = static_cast<const T *>(p.values) + lane * EPV;
-    constexpr bool kExact = std::is_same<T, float>::value;
-    float acc[kExact ? 1 : VPL][EPV];
-    dot::Dot2x2 ex[kExact ? VPL : 1][kExact ? EPV / 2 : 1];   // fp32 storage: pairs of columns
-    if constexpr (!kExact)
-#pragma unroll
-        for (int x = 0; x < VPL; ++x)
-#pragma unroll
-            for (int c = 0; c < EPV; ++c) acc[x][c] = 0.f;
+    dot::Dot2x2 ex[VPL][EPV / 2];   // pairs of columns
     if (q < E) {
         const int n = tot[q], per = (n + wpb - 1) / wpb;
         const int lo = start[q] + min(n, sub * per), hi = start[q] + min(n, (sub + 1) * per);
@@ -313,15 +386,9 @@ __global__ void __launch_bounds__(THREADS, (sizeof(T) == 4 ? 512 : 1024) / THREA
                 for (int x = 0; x < VPL; ++x) {
                     float f[EPV];
                     unpack<T>(val[u][x], f);
-                    if constexpr (kExact) {
-                        const f2 w2 = pack2(wu[u][x], wu[u][x]), n2 = pack2(-wu[u][x], -wu[u][x]);
+                    const f2 w2 = pack2(wu[u][x], wu[u][x]), n2 = pack2(-wu[u][x], -wu[u][x]);
 #pragma unroll
-                        for (int c = 0; c < EPV; c += 2) ex[x][c / 2].add(w2, n2, pack2(f[c], f[c + 1]));
-                    } else {
-#pragma unroll
-                        for (int c = 0; c < EPV; ++c)
-                            acc[x][c] = mul_add(wu[u][x], f[c], acc[x][c]);
-                    }
+                    for (int c = 0; c < EPV; c += 2) ex[x][c / 2].add(w2, n2, pack2(f[c], f[c + 1]));
                 }
         }
 #pragma unroll
@@ -329,35 +396,24 @@ __global__ void __launch_bounds__(THREADS, (sizeof(T) == 4 ? 512 : 1024) / THREA
             if (active[x])
 #pragma unroll
                 for (int c = 0; c < EPV; ++c) {
-                    R &dst = red[warp * Dv + (lane + 32 * x) * EPV + c];
-                    if constexpr (kExact) {
-                        const float2 sv = unpack2(ex[x][c / 2].s), cv = unpack2(ex[x][c / 2].c);
-                        dst = c & 1 ? make_float2(sv.y, cv.y) : make_float2(sv.x, cv.x);
-                    } else {
-                        dst = acc[x][c];
-                    }
+                    const float2 sv = unpack2(ex[x][c / 2].s), cv = unpack2(ex[x][c / 2].c);
+                    red[warp * Dv + (lane + 32 * x) * EPV + c] =
+                        c & 1 ? make_float2(sv.y, cv.y) : make_float2(sv.x, cv.x);
                 }
     }
     __syncthreads();
     const int EDv = E * Dv;
     for (int i = t; i < EDv; i += kBThreads) {
         const int qq = i / Dv, c = i - qq * Dv;
-        float sum;
-        if constexpr (kExact) {
-            Dot2 all;
-            for (int sb = 0; sb < wpb; ++sb) {
-                const float2 v = red[(qq * wpb + sb) * Dv + c];
-                Dot2 o;
-                o.s = v.x;
-                o.c = v.y;
-                all.merge(o);
-            }
-            sum = all.value_any();
-        } else {
-            sum = 0.f;
-            for (int sb = 0; sb < wpb; ++sb) sum += red[(qq * wpb + sb) * Dv + c];
+        Dot2 all;
+        for (int sb = 0; sb < wpb; ++sb) {
+            const float2 v = red[(qq * wpb + sb) * Dv + c];
+            Dot2 o;
+            o.s = v.x;
+            o.c = v.y;
+            all.merge(o);
         }
-        store_pooled<T>(d, p, b, i, sum);
+        store_pooled<T>(d, p, b, i, all.value_any());
     }
     stamp_end(p.stamp);
 }
@@ -619,39 +675,35 @@ cudaError_t configure_gather(const Dims &) {
     if (e == cudaSuccess) e = allow_padded<gather_reg_kernel<__nv_bfloat16, 1>>();
     if (e == cudaSuccess) e = allow_padded<gather_reg_kernel<__nv_bfloat16, 4>>();
     // the bucketed kernels may also be padded up to a whole SM's share (spread_smem)
-    if (e == cudaSuccess) e = allow_padded<gather_bucket_kernel<float, 512, false>>();
-    if (e == cudaSuccess) e = allow_padded<gather_bucket_kernel<__nv_bfloat16, 512, false>>();
-    if (e == cudaSuccess) e = allow_padded<gather_bucket_kernel<float, 256, false>>();
-    if (e == cudaSuccess) e = allow_padded<gather_bucket_kernel<__nv_bfloat16, 256, false>>();
-    if (e == cudaSuccess) e = allow_padded<gather_bucket_kernel<float, 512, false, 2>>();
-    if (e == cudaSuccess) e = allow_padded<gather_bucket_kernel<float, 256, false, 2>>();
+    if (e == cudaSuccess) e = allow_padded<gather_bucket_kernel<512, false>>();
+    if (e == cudaSuccess) e = allow_padded<gather_bucket_kernel<256, false>>();
+    if (e == cudaSuccess) e = allow_padded<gather_bucket_kernel<512, true>>();
+    if (e == cudaSuccess) e = allow_padded<gather_bucket_kernel<256, true>>();
+    if (e == cudaSuccess) e = allow_padded<gather_bucket_exact<512, 1>>();
+    if (e == cudaSuccess) e = allow_padded<gather_bucket_exact<256, 1>>();
+    if (e == cudaSuccess) e = allow_padded<gather_bucket_exact<512, 2>>();
+    if (e == cudaSuccess) e = allow_padded<gather_bucket_exact<256, 2>>();
     if (e == cudaSuccess) e = allow_padded<proj_kernel<float, 2, 2>>();
     if (e == cudaSuccess) e = allow_padded<proj_kernel<float, 1, 1>>();
     if (e == cudaSuccess) e = allow_padded<proj_kernel<__nv_bfloat16, 2, 2>>();
     if (e == cudaSuccess) e = allow_padded<proj_kernel<__nv_bfloat16, 1, 1>>();
-    if (e == cudaSuccess) e = allow_padded<gather_bucket_kernel<__nv_bfloat16, 512, true>>();
-    if (e == cudaSuccess) e = allow_padded<gather_bucket_kernel<__nv_bfloat16, 256, true>>();
     return e;
 }
 
 // The bucketed gather, where it serves the layer's shape (*taken).  fp32 rows
 // of 33 to 64 vectors (D_v to 256) take two vectors a lane.
-template <typename T, bool ADDR, int VPL>
-static cudaError_t launch_bucket_v(const Dims &d, const Ptrs &p, bool *taken, cudaStream_t st) {
+template <auto K512, auto K256>
+static cudaError_t launch_bucket_k(const Dims &d, const Ptrs &p, bool *taken, cudaStream_t st) {
     *taken = true;
     // spread over the SMs (see spread_smem)
-    if (d.B <= 2 * 152 && d.H * d.m <= 512) {
-        constexpr auto k = gather_bucket_kernel<T, 512, ADDR, VPL>;
-        return launch_kernel(d.pdl, k, d.B, 512,
-                             spread_smem(bucket_smem_bytes(d, 16), static_smem_of<k>(), d.B), st,
+    if (d.B <= 2 * 152 && d.H * d.m <= 512)
+        return launch_kernel(d.pdl, K512, d.B, 512,
+                             spread_smem(bucket_smem_bytes(d, 16), static_smem_of<K512>(), d.B),
+                             st, d, p);
+    if (d.H * d.m <= 256 && d.E <= 8)
+        return launch_kernel(d.pdl, K256, d.B, 256,
+                             spread_smem(bucket_smem_bytes(d, 8), static_smem_of<K256>(), d.B), st,
                              d, p);
-    }
-    if (d.H * d.m <= 256 && d.E <= 8) {
-        constexpr auto k = gather_bucket_kernel<T, 256, ADDR, VPL>;
-        return launch_kernel(d.pdl, k, d.B, 256,
-                             spread_smem(bucket_smem_bytes(d, 8), static_smem_of<k>(), d.B), st,
-                             d, p);
-    }
     *taken = false;
     return cudaSuccess;
 }
@@ -674,9 +726,17 @@ static cudaError_t launch_bucket(const Dims &d, const Ptrs &p, bool *taken, cuda
                                             32 * kGWarps, smem, st, d, p);
         }
     }
-    if (d.d_v / epv <= 32) return launch_bucket_v<T, ADDR, 1>(d, p, taken, st);
-    if constexpr (std::is_same<T, float>::value)
-        if (d.d_v / epv <= 64) return launch_bucket_v<T, ADDR, 2>(d, p, taken, st);
+    if constexpr (std::is_same<T, float>::value) {
+        if (d.d_v / epv <= 32)
+            return launch_bucket_k<gather_bucket_exact<512, 1>, gather_bucket_exact<256, 1>>(
+                d, p, taken, st);
+        if (d.d_v / epv <= 64)
+            return launch_bucket_k<gather_bucket_exact<512, 2>, gather_bucket_exact<256, 2>>(
+                d, p, taken, st);
+    } else if (d.d_v / epv <= 32) {
+        return launch_bucket_k<gather_bucket_kernel<512, ADDR>, gather_bucket_kernel<256, ADDR>>(
+            d, p, taken, st);
+    }
     return cudaSuccess;
 }
 
