@@ -44,6 +44,7 @@ using namespace tc;
 constexpr int kThreads = 256;
 constexpr int kMaxStages = 4;
 constexpr int kMaxAcc = 4;
+constexpr int kMaxSums = 8;                  // accumulators of a split chunked sum
 constexpr int kMaxSplits = 8;                // split-K CTAs per tile: one portable cluster
 constexpr size_t kSmemBudget = 225 * 1024;   // leaves room for static smem
 
@@ -118,6 +119,29 @@ template <class Op> struct MnMajor<Op, std::void_t<decltype(Op::kMnMajor)>> {
     static constexpr bool value = Op::kMnMajor;
 };
 constexpr uint32_t kMnBoxBytes = 64 * 128;   // 64 K rows of 64 bf16
+
+// An op with kChunkSums = true keeps fp32 sums at least as accurate as a chain
+// of fp32 multiply-adds.  The tensor core cuts the accumulator off at each MMA
+// instead of rounding it, so the error of a long sum grows with the number of
+// MMAs: with all of them into one accumulator, the sums of 1024 (4096) products
+// of exact three-term operands had 5 (9) times the CUDA-core projection's
+// error (share of outputs that are not the correctly rounded bf16 ones: 0.00042
+// on CUDA cores, 0.0021 so; 0.00077 and 0.0072).  Here the smaller terms' MMAs of a K block
+// come before the first term's, so that the accumulator is small for two
+// thirds of them, and an accumulator holds few K blocks; the accumulators are
+// added up rounded.  Unsplit (persistent kernel): op.sum_blocks K blocks of 64
+// each, the epilogue warps keep the sums in registers (0.0003 and 0.0003; a
+// lookup of 2048 tokens at mid_4m 68.7 -> 73.4 us, 75 with one K block each).
+// Split: the first term's blocks over all but one of the accumulators that
+// TMEM has room for (op.acc_blocks blocks each), the smaller terms of all
+// blocks in accumulator 0 (64 tokens at mid_4m: 0.00031, 0.00048 -> 0.00006;
+// 12.8 -> 13.1 us).
+template <class Op, class = void> struct ChunkSums {
+    static constexpr bool value = false;
+};
+template <class Op> struct ChunkSums<Op, std::void_t<decltype(Op::kChunkSums)>> {
+    static constexpr bool value = Op::kChunkSums;
+};
 
 // An op with kGroupEpilogue = true (the candidate-list passes: swapped)
 // reduces each group of 16 accumulator columns to one 32-bit value (group)
@@ -316,6 +340,20 @@ __global__ void __launch_bounds__(kThreads, 1)
 #pragma unroll
             for (int j = 0; j < NSPLIT; ++j) bd0[j] = kMn ? desc_mn_sw128(sa + a_bytes + j * b_bytes)
                              : desc_k_sw128(sa + a_bytes + j * b_bytes);
+            if constexpr (ChunkSums<Op>::value) {
+                static_assert(!kSwap, "split ops keep the outputs on the lanes");
+#pragma unroll
+                for (int j = NSPLIT - 1; j >= 0; --j) {
+                    const int a = j ? 0 : 1 + it / op.acc_blocks;
+                    const uint32_t dt = tmem + (uint32_t)(a * acc_n);
+#pragma unroll
+                    for (int k16 = 0; k16 < kBlockK / 16; ++k16) {
+                        mma_bf16(dt, ad0 + kStep * k16, bd0[j] + kStep * k16, idesc,
+                                 started >> a & 1u);
+                        started |= 1u << a;
+                    }
+                }
+            } else
 #pragma unroll
             for (int k16 = 0; k16 < kBlockK / 16; ++k16) {
                 const int kg = (t.kb0 + it) * kBlockK + k16 * 16;
@@ -381,7 +419,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         __syncthreads();
         if (warp == 0) tmem_dealloc(tmem, ncols);
     } else {
-        // Split-K through distributed shared memory (one accumulator): each
+        // Split-K through distributed shared memory: each
         // CTA stages its partial; once every CTA of the cluster has staged
         // its own (so that every ring is drained), it sends slice j to CTA j
         // with one bulk copy into j's receive slot for it (completing bytes
@@ -396,6 +434,18 @@ __global__ void __launch_bounds__(kThreads, 1)
             uint32_t r[32];
             tmem_ld32_nowait(lane_base + (uint32_t)c0, r);
             tmem_ld_wait();
+            if constexpr (ChunkSums<Op>::value) {   // the accumulators that were used
+                const int used = 1 + (t.nkb + op.acc_blocks - 1) / op.acc_blocks;
+#pragma unroll 1
+                for (int a = 1; a < used; ++a) {
+                    uint32_t ra[32];
+                    tmem_ld32_nowait(lane_base + (uint32_t)(a * acc_n + c0), ra);
+                    tmem_ld_wait();
+#pragma unroll
+                    for (int i = 0; i < 32; ++i)
+                        r[i] = __float_as_uint(__uint_as_float(r[i]) + __uint_as_float(ra[i]));
+                }
+            }
 #pragma unroll
             for (int g = 0; g < 8; ++g) {
                 const int c = c0 + 4 * g;
@@ -579,6 +629,43 @@ __global__ void __launch_bounds__(persistent_threads<Op>(), 1)
             const uint32_t idesc = kSwap ? idesc_bf16_f32(n_tile, kA) : idesc_bf16_f32(kTileM, n_tile);
             const int acc_n = acc_cols_of(op);
             int it = 0, lt = 0;
+            if constexpr (ChunkSums<Op>::value) {   // a buffer per op.sum_blocks K blocks
+                bool ok = true;
+                for (int i = blockIdx.x; ok && i < tiles && !abort_flag; i += gridDim.x) {
+                    const Tile t = tile_of(i);
+                    for (int kb = 0; kb < t.nkb; ++kb, ++it) {
+                        const bool first = (kb & (op.sum_blocks - 1)) == 0;
+                        const int buf = lt & 1, s = it % kStages;
+                        if ((first && lt >= 2 && !mbar_wait(&tempty[buf], ((lt >> 1) - 1) & 1)) ||
+                            !mbar_wait(&full[s], (it / kStages) & 1)) {
+                            fail();
+                            ok = false;
+                            break;
+                        }
+                        tc_fence_after();
+                        const uint32_t dt = tmem + (uint32_t)buf * buf_cols;
+                        const uint32_t sa = smem_u32(ring + (size_t)s * stage_bytes);
+                        const uint64_t ad0 = desc_k_sw128(sa);
+#pragma unroll
+                        for (int j = NSPLIT - 1; j >= 0; --j) {   // the smaller terms first
+                            const uint64_t bd0 = desc_k_sw128(sa + a_bytes + j * b_bytes);
+#pragma unroll
+                            for (int k16 = 0; k16 < kBlockK / 16; ++k16) {
+                                const uint32_t more = !first || j < NSPLIT - 1 || k16 > 0;
+                                if constexpr (kSwap)
+                                    mma_bf16(dt, bd0 + 2 * k16, ad0 + 2 * k16, idesc, more);
+                                else
+                                    mma_bf16(dt, ad0 + 2 * k16, bd0 + 2 * k16, idesc, more);
+                            }
+                        }
+                        mma_commit(&empty[s]);
+                        if (((kb + 1) & (op.sum_blocks - 1)) == 0 || kb + 1 == t.nkb) {
+                            mma_commit(&tfull[buf]);
+                            ++lt;
+                        }
+                    }
+                }
+            } else
             for (int i = blockIdx.x; i < tiles && !abort_flag; i += gridDim.x, ++lt) {
                 const Tile t = tile_of(i);
                 const int buf = lt & 1;
@@ -644,6 +731,58 @@ __global__ void __launch_bounds__(persistent_threads<Op>(), 1)
         const int quad = warp & 3, grp = (warp - 2) >> 2;
         const int row = quad * 32 + lane;
         int lt = 0;
+        if constexpr (ChunkSums<Op>::value) {
+            static_assert(kEG == 4, "at most 256 columns, two chunks of 32 a warp");
+            const int acc_n = acc_cols_of(op);
+            bool ok = true;
+            for (int i = blockIdx.x; i < tiles && !abort_flag; i += gridDim.x) {
+                const Tile t = tile_of(i);
+                float sum[2][32];
+#pragma unroll
+                for (int h = 0; h < 2; ++h)
+#pragma unroll
+                    for (int e = 0; e < 32; ++e) sum[h][e] = 0.f;
+#pragma unroll 1
+                for (int kb = 0; kb < t.nkb; kb += op.sum_blocks, ++lt) {
+                    const int buf = lt & 1;
+                    if (!mbar_wait(&tfull[buf], (lt >> 1) & 1)) {
+                        if (lane == 0) fail();
+                        ok = false;
+                        break;
+                    }
+                    tc_fence_after();
+                    const uint32_t lane_base =
+                        tmem + (uint32_t)buf * buf_cols + ((uint32_t)(quad * 32) << 16);
+#pragma unroll
+                    for (int h = 0; h < 2; ++h) {
+                        const int c0 = (grp + h * kEG) * 32;
+                        if (c0 >= acc_n) break;
+#pragma unroll
+                        for (int z = 0; z < 32; z += 16) {
+                            float r[16];
+                            tmem_ld16(lane_base + (uint32_t)(c0 + z), r);
+#pragma unroll
+                            for (int e = 0; e < 16; ++e) sum[h][z + e] += r[e];
+                        }
+                    }
+                    tc_fence_before();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(&tempty[buf]);
+                }
+                if (!ok) break;
+#pragma unroll
+                for (int h = 0; h < 2; ++h)
+#pragma unroll
+                    for (int half = 0; half < 2; ++half) {
+                        const int c = (grp + h * kEG) * 32 + half * 16;
+                        if (c >= acc_n) break;
+                        float v[kMaxAcc][16];
+#pragma unroll
+                        for (int q = 0; q < 16; ++q) v[0][q] = sum[h][half * 16 + q];
+                        op.store(t, row, c, v, 0u);
+                    }
+            }
+        } else
         for (int i = blockIdx.x; i < tiles && !abort_flag; i += gridDim.x, ++lt) {
             const Tile t = tile_of(i);
             const int buf = lt & 1;
@@ -1022,6 +1161,18 @@ struct ProjRowsOp {
     }
 };
 
+// The projection of the lookup-reduce: three exact terms of the pooled rows,
+// sums as accurate as plain fp32 ones (kChunkSums).
+struct ProjSumOp : ProjOp {
+    static constexpr bool kChunkSums = true;
+    int sum_blocks;   // unsplit: K blocks an accumulator holds
+    int acc_blocks;   // split: K blocks an accumulator of the first term holds
+};
+template <int AR> struct ProjRowsSumOp : ProjRowsOp<AR> {
+    static constexpr bool kChunkSums = true;
+    int sum_blocks;   // K blocks an accumulator holds
+};
+
 // The backward's dacc = W_p g (the projectors as stored, [E D_v][D'_v], are
 // the K-major A operand; the gradient rows g [B][D'_v] the B operand): fp32
 // rows dacc[B][E D_v], unsplit.
@@ -1195,6 +1346,8 @@ static uint32_t buf_cols_of(int n_acc, int n_tile) {
 // does not apply.
 template <int NSPLIT, class Op>
 static bool persistent_ok(dim3 grid, const Op &op) {
+    // (chunked sums: the kernel for every unsplit grid)
+    if (ChunkSums<Op>::value) return op.cluster_splits_host() == 1;
     const uint32_t bc = buf_cols_of(op.n_acc, acc_cols_of(op));
     return grid.z >= 1 && op.cluster_splits_host() == 1 &&
            (int)(grid.x * grid.y * grid.z) > sm_count() && 2 * bc <= 512 &&
@@ -1211,10 +1364,13 @@ static cudaError_t launch_gemm_persistent(dim3 grid, const CUtensorMap &a0, cons
     const size_t smem = 1024 + (size_t)op.stages * stage_bytes_of(NSPLIT, op.n_tile, kA);
     const int tiles = (int)(grid.x * grid.y * grid.z);
     const int ctas = tiles < sm_count() ? tiles : sm_count();
+    // both buffers are one TMEM allocation, a power of two (persistent_ok asks
+    // for that; chunked sums, which have no other kernel, round up to it)
+    uint32_t buf = buf_cols_of(op.n_acc, acc_cols_of(op));
+    if (ChunkSums<Op>::value) buf = tmem_cols_for(2 * buf_cols_of(1, acc_cols_of(op))) / 2;
     return launch_kernel(pdl, tc_gemm_persistent<NSPLIT, Op>, dim3(ctas),
                          persistent_threads<Op>(), smem, st, a0,
-                         a1, b, op, (int)grid.x, (int)grid.y, tiles,
-                         buf_cols_of(op.n_acc, acc_cols_of(op)), probe);
+                         a1, b, op, (int)grid.x, (int)grid.y, tiles, buf, probe);
 }
 
 // grid.z = the split count (S1, S9; also the cluster's z extent when > 1) or
@@ -1225,8 +1381,9 @@ static cudaError_t launch_gemm(dim3 grid, const CUtensorMap &a0, const CUtensorM
                                cudaStream_t st, int probe = 0) {
     if (persistent_ok<NSPLIT>(grid, op))
         return launch_gemm_persistent<NSPLIT>(grid, a0, a1, b, op, nkb, pdl, st, probe);
-    // the split-K epilogue adds up one accumulator
-    if (op.cluster_splits_host() > 1 && op.n_acc != 1) return cudaErrorInvalidValue;
+    // the split-K epilogue adds up one accumulator (or, chunked, all of them)
+    if (!ChunkSums<Op>::value && op.cluster_splits_host() > 1 && op.n_acc != 1)
+        return cudaErrorInvalidValue;
     constexpr int kA = ARows<Op>::value;
     op.stages = stages_for(NSPLIT, op.n_tile, nkb, kA);
     const size_t ring = (size_t)op.stages * stage_bytes_of(NSPLIT, op.n_tile, kA);
@@ -1237,14 +1394,15 @@ static cudaError_t launch_gemm(dim3 grid, const CUtensorMap &a0, const CUtensorM
                          kThreads, smem, st, a0, a1, b, op, probe);
 }
 
+template <int NSPLIT, class Op> static cudaError_t allow_persistent() {
+    return cudaFuncSetAttribute(tc_gemm_persistent<NSPLIT, Op>,
+                                cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBudget);
+}
 template <int NSPLIT, class Op> static cudaError_t allow_smem() {
-    cudaError_t e = cudaFuncSetAttribute(tc_gemm_kernel<NSPLIT, Op>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)kSmemBudget);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(tc_gemm_persistent<NSPLIT, Op>,
-                                 cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBudget);
-    return e;
+    const cudaError_t e = cudaFuncSetAttribute(tc_gemm_kernel<NSPLIT, Op>,
+                                               cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                               (int)kSmemBudget);
+    return e == cudaSuccess ? allow_persistent<NSPLIT, Op>() : e;
 }
 
 cudaError_t configure_tc() {
@@ -1254,11 +1412,11 @@ cudaError_t configure_tc() {
     if (e == cudaSuccess) e = allow_smem<3, ScoreListOp<kListGroupMax>>();
     if (e == cudaSuccess) e = allow_smem<3, ScoreListOp<kListCandidates>>();
     if (e == cudaSuccess) e = allow_smem<2, ProjOp>();
-    if (e == cudaSuccess) e = allow_smem<3, ProjOp>();
+    if (e == cudaSuccess) e = allow_smem<3, ProjSumOp>();
     if (e == cudaSuccess) e = allow_smem<2, ProjRowsOp<128>>();
-    if (e == cudaSuccess) e = allow_smem<3, ProjRowsOp<128>>();
     if (e == cudaSuccess) e = allow_smem<2, ProjRowsOp<256>>();
-    if (e == cudaSuccess) e = allow_smem<3, ProjRowsOp<256>>();
+    if (e == cudaSuccess) e = allow_persistent<3, ProjRowsSumOp<128>>();
+    if (e == cudaSuccess) e = allow_persistent<3, ProjRowsSumOp<256>>();
     if (e == cudaSuccess) e = allow_smem<1, DaccOp>();
     if (e == cudaSuccess) e = allow_smem<2, DwOp>();
     if (e == cudaSuccess)
@@ -1444,10 +1602,15 @@ static int proj_rows(const Dims &d) {
 }
 uint32_t proj_token_box(const Dims &d) { return proj_rows(d) ? kTileM : (uint32_t)d.p_ntile; }
 
-template <int AR>
-static cudaError_t launch_proj_rows(const Dims &d, const Ptrs &p, const TcMaps &mp, int acc_terms,
+// K blocks an accumulator of a chunked sum holds: two from 1024 products on,
+// where a chain of multiply-adds has gathered more error than 16 MMAs leave.
+static int sum_blocks_of(int kb) { return kb >= 16 ? 2 : 1; }
+
+template <int NSPLIT, class Op>
+static cudaError_t launch_proj_rows(const Dims &d, const Ptrs &p, const TcMaps &mp,
                                     cudaStream_t st) {
-    ProjRowsOp<AR> op;
+    constexpr int AR = Op::kARows;
+    Op op;
     op.stamp = p.stamp;
     op.n_tile = kTileM;
     op.n_acc = 1;
@@ -1459,27 +1622,27 @@ static cudaError_t launch_proj_rows(const Dims &d, const Ptrs &p, const TcMaps &
     op.kb_total = (d.E * d.d_v + kBlockK - 1) / kBlockK;
     op.out = static_cast<__nv_bfloat16 *>(p.out);
     op.vec = d.d_out % 8 == 0 && ((uintptr_t)p.out & 15) == 0;
+    if constexpr (ChunkSums<Op>::value) op.sum_blocks = sum_blocks_of(op.kb_total);
     dim3 grid((d.d_out + AR - 1) / AR, (d.B + kTileM - 1) / kTileM, 1);
-    return acc_terms == 3
-               ? launch_gemm<3>(grid, mp.w_pt, mp.w_pt, mp.acc, op, op.kb_total, d.pdl, st)
-               : launch_gemm<2>(grid, mp.w_pt, mp.w_pt, mp.acc, op, op.kb_total, d.pdl, st);
+    if constexpr (ChunkSums<Op>::value)
+        return launch_gemm_persistent<NSPLIT>(grid, mp.w_pt, mp.w_pt, mp.acc, op, op.kb_total,
+                                              d.pdl, st, 0);
+    else
+        return launch_gemm<NSPLIT>(grid, mp.w_pt, mp.w_pt, mp.acc, op, op.kb_total, d.pdl, st);
 }
 
-cudaError_t launch_proj_tc(const Dims &d, const Ptrs &p, const TcMaps &mp, int acc_terms,
-                           cudaStream_t st) {
-    if (d.p_splits > kMaxSplits) return cudaErrorInvalidValue;
-    if (const int ar = proj_rows(d))
-        return ar == 256 ? launch_proj_rows<256>(d, p, mp, acc_terms, st)
-                         : launch_proj_rows<128>(d, p, mp, acc_terms, st);
-    ProjOp op;
+// The pooled rows are two or three bf16 terms ([B][terms][E D_v]): all
+// multiply each projector tile into fp32 accumulators, so the operand
+// carries the pooled value to 2^-16 relative (two) or exactly (three)
+// instead of one rounding.
+template <int NSPLIT, class Op>
+static cudaError_t launch_proj_op(const Dims &d, const Ptrs &p, const TcMaps &mp,
+                                  cudaStream_t st) {
+    Op op;
     op.stamp = p.stamp;
     op.n_tile = d.p_ntile ? d.p_ntile : tc_n_tile(d.B, 1);
     op.n_acc = 1;
     op.acc_chunk = 1 << 30;
-    // the pooled rows are two or three bf16 terms ([B][terms][E D_v]): all
-    // multiply each projector tile into one fp32 accumulator, so the operand
-    // carries the pooled value to 2^-16 relative (two) or exactly (three)
-    // instead of one rounding
     op.b_split_stride = d.E * d.d_v;
     op.err = p.err;
     op.B = d.B;
@@ -1489,8 +1652,29 @@ cudaError_t launch_proj_tc(const Dims &d, const Ptrs &p, const TcMaps &mp, int a
     op.out = static_cast<__nv_bfloat16 *>(p.out);
     dim3 grid((d.d_out + kTileM - 1) / kTileM, (d.B + op.n_tile - 1) / op.n_tile, op.splits);
     const int per = (op.kb_total + op.splits - 1) / op.splits;
-    return acc_terms == 3 ? launch_gemm<3>(grid, mp.w_pt, mp.w_pt, mp.acc, op, per, d.pdl, st)
-                          : launch_gemm<2>(grid, mp.w_pt, mp.w_pt, mp.acc, op, per, d.pdl, st);
+    if constexpr (ChunkSums<Op>::value) {
+        // as many accumulators as TMEM's 512 columns hold (reads cover whole
+        // 32 columns), one of them for the smaller terms
+        const int room = 1 + (512 - (op.n_tile + 31) / 32 * 32) / op.n_tile;
+        const int hi = (room < kMaxSums ? room : kMaxSums) - 1;
+        op.sum_blocks = sum_blocks_of(per);
+        op.acc_blocks = (per + hi - 1) / hi;
+        op.n_acc = 1 + (per + op.acc_blocks - 1) / op.acc_blocks;
+    }
+    return launch_gemm<NSPLIT>(grid, mp.w_pt, mp.w_pt, mp.acc, op, per, d.pdl, st);
+}
+
+cudaError_t launch_proj_tc(const Dims &d, const Ptrs &p, const TcMaps &mp, int acc_terms,
+                           cudaStream_t st) {
+    if (d.p_splits > kMaxSplits) return cudaErrorInvalidValue;
+    const int ar = proj_rows(d);
+    if (acc_terms == 3)
+        return ar == 256   ? launch_proj_rows<3, ProjRowsSumOp<256>>(d, p, mp, st)
+               : ar == 128 ? launch_proj_rows<3, ProjRowsSumOp<128>>(d, p, mp, st)
+                           : launch_proj_op<3, ProjSumOp>(d, p, mp, st);
+    return ar == 256   ? launch_proj_rows<2, ProjRowsOp<256>>(d, p, mp, st)
+           : ar == 128 ? launch_proj_rows<2, ProjRowsOp<128>>(d, p, mp, st)
+                       : launch_proj_op<2, ProjOp>(d, p, mp, st);
 }
 
 }  // namespace um
