@@ -1012,12 +1012,16 @@ ultramem_status ultramem_lookup_reduce_backward(ultramem_layer *L, const int64_t
     if (dw_proj && d.has_proj && L->tc && L->dacc_tc && B >= kLongBackward &&
         L->cfg.d_out % 8 == 0) {
         const int kd = d.E * d.d_v;
+        // whole 16-byte rows of tokens enter as two terms hi + lo, as the
+        // transposed operands below do; other counts, whose products the CUDA
+        // cores take from the fp32 rows, as three exact ones
+        const int terms = B % 8 == 0 ? 2 : 3;
         CUtensorMap am, gm;
         Ptrs pg = p;
-        pg.acc_bf = L->ws.acc_bf;   // [B][2][E D_v]
-        pg.acc_terms = 2;
+        pg.acc_bf = L->ws.acc_bf;   // [B][terms][E D_v]
+        pg.acc_terms = terms;
         bool gathered = false;
-        if (um::tc_encode(&am, L->ws.acc_bf, 2ull * kd, (uint64_t)B, 1, 64, 2) &&
+        if (um::tc_encode(&am, L->ws.acc_bf, (uint64_t)terms * kd, (uint64_t)B, 1, 64, 2) &&
             um::tc_encode(&gm, g, (uint64_t)L->cfg.d_out, (uint64_t)B, 1, 64, 2)) {
             if ((e = um::launch_gather_addresses(d, pg, &gathered, st)) != cudaSuccess)
                 return from_cuda(e);
@@ -1029,7 +1033,7 @@ ultramem_status ultramem_lookup_reduce_backward(ultramem_layer *L, const int64_t
                 n = 2;
             }
             d.pdl = 1;
-            if ((e = um::launch_dw_mn(d, gm, am, dw_proj, L->ws.err, st)) != cudaSuccess)
+            if ((e = um::launch_dw_mn(d, gm, am, terms, dw_proj, L->ws.err, st)) != cudaSuccess)
                 return from_cuda(e);
             ++n;
             chained = true;

@@ -143,10 +143,10 @@ cudaError_t launch_dacc_tc(const Dims &d, const CUtensorMap &w_p, const CUtensor
 // bf16 terms [E D_v][2 B] (hi in columns [0, B), lo in [B, 2 B))
 cudaError_t launch_dw_tc(const Dims &d, const CUtensorMap &g_t, const CUtensorMap &acc_t2,
                          float *dW, int *err, cudaStream_t st);
-// the same from g [B][D'_v] and the pooled rows' terms [B][2 E D_v] (maps with
-// boxes of 64 rows)
-cudaError_t launch_dw_mn(const Dims &d, const CUtensorMap &g, const CUtensorMap &acc2, float *dW,
-                         int *err, cudaStream_t st);
+// the same from g [B][D'_v] and the pooled rows' two or three terms
+// [B][terms E D_v] (maps with boxes of 64 rows)
+cudaError_t launch_dw_mn(const Dims &d, const CUtensorMap &g, const CUtensorMap &acc, int terms,
+                         float *dW, int *err, cudaStream_t st);
 // tokens a TMA box of the dacc contraction's map g covers
 int dacc_token_box(const Dims &d);
 // dst[c][r] = src[r][c], rows x cols bf16; row strides ld_src / ld_dst in

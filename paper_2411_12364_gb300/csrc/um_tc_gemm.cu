@@ -110,8 +110,8 @@ template <class Op> struct ARows<Op, std::void_t<decltype(Op::kARows)>> {
 
 // An op with kMnMajor = true reads operands whose rows run along K (the
 // contraction sums over the rows of both): boxes of 64 K rows x 64 columns,
-// MN-major tiles of the MMA.  No transposed copies.  (One-CTA-per-tile
-// kernel only; n_tile a multiple of 64.)
+// MN-major tiles of the MMA.  No transposed copies.  (n_tile a multiple of 64;
+// in the persistent kernel with kChunkSums only.)
 template <class Op, class = void> struct MnMajor {
     static constexpr bool value = false;
 };
@@ -601,6 +601,17 @@ __global__ void __launch_bounds__(persistent_threads<Op>(), 1)
                     uint8_t *sa = ring + (size_t)s * stage_bytes;
                     mbar_arrive_expect_tx(&full[s], stage_bytes);
                     const int kx = (t.kb0 + kb) * kBlockK;
+                    if constexpr (MnMajor<Op>::value) {
+#pragma unroll
+                        for (int x = 0; x < kTileM / 64; ++x)
+                            tma_load_2d(sa + x * kMnBoxBytes, mapA, &full[s], t.m0 + 64 * x, kx);
+#pragma unroll
+                        for (int j = 0; j < NSPLIT; ++j)
+                            for (int x = 0; x < n_tile / 64; ++x)
+                                tma_load_2d(sa + a_bytes + j * b_bytes + x * kMnBoxBytes, &mapB,
+                                            &full[s], j * op.b_split_stride + t.n0 + 64 * x, kx);
+                        continue;
+                    }
 #pragma unroll
                     for (int ab = 0; ab < kA / kTileM; ++ab) {
                         uint8_t *sab = sa + ab * kTileABytes;
@@ -626,7 +637,11 @@ __global__ void __launch_bounds__(persistent_threads<Op>(), 1)
         if (lane == 0) {
             // MMA issuer
             constexpr bool kSwap = SwapAB<Op>::value;
-            const uint32_t idesc = kSwap ? idesc_bf16_f32(n_tile, kA) : idesc_bf16_f32(kTileM, n_tile);
+            constexpr bool kMn = MnMajor<Op>::value;
+            const uint32_t idesc =
+                (kSwap ? idesc_bf16_f32(n_tile, kA) : idesc_bf16_f32(kTileM, n_tile)) |
+                (kMn ? kIdescMnMajor : 0u);
+            constexpr int kStep = kMn ? 16 * 128 >> 4 : 32 >> 4;   // per 16 K, as above
             const int acc_n = acc_cols_of(op);
             int it = 0, lt = 0;
             if constexpr (ChunkSums<Op>::value) {   // a buffer per op.sum_blocks K blocks
@@ -645,17 +660,18 @@ __global__ void __launch_bounds__(persistent_threads<Op>(), 1)
                         tc_fence_after();
                         const uint32_t dt = tmem + (uint32_t)buf * buf_cols;
                         const uint32_t sa = smem_u32(ring + (size_t)s * stage_bytes);
-                        const uint64_t ad0 = desc_k_sw128(sa);
+                        const uint64_t ad0 = kMn ? desc_mn_sw128(sa) : desc_k_sw128(sa);
 #pragma unroll
                         for (int j = NSPLIT - 1; j >= 0; --j) {   // the smaller terms first
-                            const uint64_t bd0 = desc_k_sw128(sa + a_bytes + j * b_bytes);
+                            const uint32_t sb = sa + a_bytes + j * b_bytes;
+                            const uint64_t bd0 = kMn ? desc_mn_sw128(sb) : desc_k_sw128(sb);
 #pragma unroll
                             for (int k16 = 0; k16 < kBlockK / 16; ++k16) {
                                 const uint32_t more = !first || j < NSPLIT - 1 || k16 > 0;
                                 if constexpr (kSwap)
-                                    mma_bf16(dt, bd0 + 2 * k16, ad0 + 2 * k16, idesc, more);
+                                    mma_bf16(dt, bd0 + kStep * k16, ad0 + kStep * k16, idesc, more);
                                 else
-                                    mma_bf16(dt, ad0 + 2 * k16, bd0 + 2 * k16, idesc, more);
+                                    mma_bf16(dt, ad0 + kStep * k16, bd0 + kStep * k16, idesc, more);
                             }
                         }
                         mma_commit(&empty[s]);
@@ -1259,6 +1275,13 @@ struct DwOp {
 struct DwMnOp : DwOp {
     static constexpr bool kMnMajor = true;
 };
+// From three exact terms, with sums as accurate as plain fp32 ones.
+struct DwMnSumOp : DwOp {
+    static constexpr bool kMnMajor = true;
+    static constexpr bool kChunkSums = true;
+    static constexpr int kEpiWarps = 16;
+    int sum_blocks;   // K blocks an accumulator holds
+};
 
 // dst[c][r] = src[r][c] for a rows x cols bf16 matrix (32 x 32 tiles), with
 // row strides ld_src (>= cols) and ld_dst (>= rows) in elements
@@ -1422,6 +1445,7 @@ cudaError_t configure_tc() {
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(tc_gemm_kernel<2, DwMnOp>,
                                  cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBudget);
+    if (e == cudaSuccess) e = allow_persistent<3, DwMnSumOp>();
     return e;
 }
 
@@ -1442,9 +1466,10 @@ cudaError_t launch_dw_tc(const Dims &d, const CUtensorMap &g_t, const CUtensorMa
     return launch_gemm<2>(grid, g_t, g_t, acc_t2, op, op.kb_total, false, st);
 }
 
-cudaError_t launch_dw_mn(const Dims &d, const CUtensorMap &g, const CUtensorMap &acc2, float *dW,
-                         int *err, cudaStream_t st) {
-    DwMnOp op;
+template <int NSPLIT, class Op>
+static cudaError_t launch_dw_mn_op(const Dims &d, const CUtensorMap &g, const CUtensorMap &acc,
+                                   float *dW, int *err, cudaStream_t st) {
+    Op op;
     op.stamp = nullptr;
     op.M = d.d_out;
     op.N = d.E * d.d_v;
@@ -1459,15 +1484,25 @@ cudaError_t launch_dw_mn(const Dims &d, const CUtensorMap &g, const CUtensorMap 
         op.n_tile /= 2;
     op.n_acc = 1;
     op.acc_chunk = 1 << 30;
-    op.b_split_stride = op.N;   // the lo term follows the hi term in a row
+    op.b_split_stride = op.N;   // the next term follows in a row
     op.err = err;
     op.kb_total = (d.B + kBlockK - 1) / kBlockK;
     op.out = dW;
     dim3 grid(m_tiles, (op.N + op.n_tile - 1) / op.n_tile, 1);
-    op.stages = stages_for(2, op.n_tile, op.kb_total);
-    const size_t smem = 1024 + (size_t)op.stages * stage_bytes_of(2, op.n_tile);
-    return launch_kernel(d.pdl, 1u, tc_gemm_kernel<2, DwMnOp>, grid, kThreads, smem, st, g, g,
-                         acc2, op, 0);
+    if constexpr (ChunkSums<Op>::value) {
+        op.sum_blocks = 1;   // a tile's sums are few: the accuracy costs nothing
+        return launch_gemm_persistent<NSPLIT>(grid, g, g, acc, op, op.kb_total, d.pdl, st, 0);
+    } else {
+        op.stages = stages_for(NSPLIT, op.n_tile, op.kb_total);
+        const size_t smem = 1024 + (size_t)op.stages * stage_bytes_of(NSPLIT, op.n_tile);
+        return launch_kernel(d.pdl, 1u, tc_gemm_kernel<NSPLIT, Op>, grid, kThreads, smem, st, g,
+                             g, acc, op, 0);
+    }
+}
+cudaError_t launch_dw_mn(const Dims &d, const CUtensorMap &g, const CUtensorMap &acc, int terms,
+                         float *dW, int *err, cudaStream_t st) {
+    return terms == 3 ? launch_dw_mn_op<3, DwMnSumOp>(d, g, acc, dW, err, st)
+                      : launch_dw_mn_op<2, DwMnOp>(d, g, acc, dW, err, st);
 }
 
 // tokens a tile of the dacc contraction: 128 where 256 would leave SMs idle

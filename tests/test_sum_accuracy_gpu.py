@@ -1,4 +1,4 @@
-"""The tensor-core sums of the lookup-reduce against a chain
+"""The tensor-core sums of the lookup-reduce and its backward against a chain
 of fp32 multiply-adds: their error against 64 bits is no larger than such a
 chain's, at the sizes where the kernels split the sum differently (over CTAs,
 over accumulators, over K blocks in the epilogue's registers).
@@ -63,3 +63,18 @@ def test_projection_sums(B, d_v, d_out, gpu_lib):
     got = int((out != right).sum())
     # both counts are of rare independent events: three standard deviations
     assert got <= chain + 3 * (2 * chain) ** 0.5 + 3, (got, chain)
+
+
+@pytest.mark.parametrize("B", [513, 1001, 2047, 4095])
+def test_projector_gradient_sums(B, gpu_lib):
+    """dW_p of token counts that are not whole 16-byte rows: rms error."""
+    cfg, w, idx, wt, acc, gen = _layer(B, 256, 256)
+    g = torch.randn((B, 256), generator=gen, device="cuda").bfloat16()
+    layer = binding.UltraMemLayer(cfg, w, B)
+    dwp = layer.lookup_reduce_backward(idx, wt, g)[2][0]
+    assert layer.check() == binding.OK
+    layer.close()
+    right = acc.double().T @ g.double()
+    rms = (dwp.double() - right).square().mean().sqrt()
+    chain = (_chain(acc, g).double() - right).square().mean().sqrt()
+    assert rms <= chain, (float(rms), float(chain))
