@@ -849,6 +849,7 @@ ultramem_status ultramem_create(const ultramem_config *cfg, const ultramem_weigh
             ok = ok && um::tc_encode(&L->maps.w_pt, ws.w_pt, kd, cfg->d_out, 1, 128, 2);
             // the projectors as stored, for the backward's dacc = W_p g (when
             // D'_v rows are whole 16-byte vectors; else the CUDA-core path)
+            L->maps.w_pt_rows = ws.w_pt;
             L->dacc_tc = um::tc_encode(&L->maps.w_p, w->w_proj, cfg->d_out, kd, 1, 128, 2);
         } else {
             L->maps.w_pt = L->maps.w_q;
@@ -1033,7 +1034,8 @@ ultramem_status ultramem_lookup_reduce_backward(ultramem_layer *L, const int64_t
                 n = 2;
             }
             d.pdl = 1;
-            if ((e = um::launch_dw_mn(d, gm, am, terms, dw_proj, L->ws.err, st)) != cudaSuccess)
+            if ((e = um::launch_dw_mn(d, gm, am, g, L->ws.acc_bf, terms, dw_proj, L->ws.err,
+                                      st)) != cudaSuccess)
                 return from_cuda(e);
             ++n;
             chained = true;

@@ -110,6 +110,7 @@ struct TcMaps {
     CUtensorMap qs_t;    // the split queries with 128-token boxes (candidate lists)
     CUtensorMap xs;      // the convolved input's three bf16 terms [B][3 D_i]
     CUtensorMap w_p;     // the projectors as stored, [E D_v][D'_v] (backward's A)
+    const __nv_bfloat16 *w_pt_rows;   // what w_pt maps, [D'_v][E D_v]
 };
 
 bool tc_init();
@@ -144,9 +145,10 @@ cudaError_t launch_dacc_tc(const Dims &d, const CUtensorMap &w_p, const CUtensor
 cudaError_t launch_dw_tc(const Dims &d, const CUtensorMap &g_t, const CUtensorMap &acc_t2,
                          float *dW, int *err, cudaStream_t st);
 // the same from g [B][D'_v] and the pooled rows' two or three terms
-// [B][terms E D_v] (maps with boxes of 64 rows)
-cudaError_t launch_dw_mn(const Dims &d, const CUtensorMap &g, const CUtensorMap &acc, int terms,
-                         float *dW, int *err, cudaStream_t st);
+// [B][terms E D_v] (maps with boxes of 64 rows, and the rows themselves)
+cudaError_t launch_dw_mn(const Dims &d, const CUtensorMap &g, const CUtensorMap &acc,
+                         const void *g_rows, const __nv_bfloat16 *acc_rows, int terms, float *dW,
+                         int *err, cudaStream_t st);
 // tokens a TMA box of the dacc contraction's map g covers
 int dacc_token_box(const Dims &d);
 // dst[c][r] = src[r][c], rows x cols bf16; row strides ld_src / ld_dst in

@@ -497,6 +497,10 @@ __global__ void __launch_bounds__(kThreads, 1)
                 }
             }
             op.store_sums(t, it % kTileM, (int)me * per + 4 * (it / kTileM), sums);
+            if constexpr (ChunkSums<Op>::value) {
+                const float z = (sums[0] + sums[1]) * 0.f + (sums[2] + sums[3]) * 0.f;
+                if (!(z == 0.f)) op.again(t, it % kTileM, (int)me * per + 4 * (it / kTileM), 4);
+            }
         }
         cluster_wait();
     }
@@ -797,6 +801,14 @@ __global__ void __launch_bounds__(persistent_threads<Op>(), 1)
                         for (int q = 0; q < 16; ++q) v[0][q] = sum[h][half * 16 + q];
                         op.store(t, row, c, v, 0u);
                     }
+                float z = 0.f;   // a NaN when a sum is not finite
+#pragma unroll
+                for (int h = 0; h < 2; ++h)
+#pragma unroll
+                    for (int e = 0; e < 32; ++e) z = fmaf(sum[h][e], 0.f, z);
+                if (!(z == 0.f))
+#pragma unroll 1
+                    for (int c0 = grp * 32; c0 < acc_n; c0 += 32 * kEG) op.again(t, row, c0, 32);
             }
         } else
         for (int i = blockIdx.x; i < tiles && !abort_flag; i += gridDim.x, ++lt) {
@@ -1177,16 +1189,58 @@ struct ProjRowsOp {
     }
 };
 
+// Sums of products again, by plain fp32 multiply-adds, where `out` (cnt of them,
+// so far apart) holds a NaN: sum e is over i < n of a_i w_i, a_i given as its
+// three terms, `term` elements apart.  Where a_i w_i is infinite the products
+// of a_i's terms are infinite or, for a term that is zero, a NaN; so a chunked
+// sum that comes out a NaN is taken from here (where it may be one as well).
+template <typename O>
+__device__ __noinline__ void sums_again(O *out, int64_t out_step, const __nv_bfloat16 *a,
+                                        int64_t a_step, const __nv_bfloat16 *w, int64_t w_step,
+                                        int cnt, int64_t sa, int64_t term, int64_t sw, int n) {
+#pragma unroll 1
+    for (int e = 0; e < cnt; ++e, out += out_step, a += a_step, w += w_step) {
+        const float had = to_f(*out);
+        if (had == had) continue;
+        float s = 0.f;
+#pragma unroll 1
+        for (int i = 0; i < n && s == s; ++i) {
+            const __nv_bfloat16 *t = a + i * sa;
+            const float v = to_f(t[0]) + (to_f(t[term]) + to_f(t[2 * term]));   // exact
+            s = fmaf(v, to_f(w[i * sw]), s);
+        }
+        *out = from_f<O>(s);
+    }
+}
+
 // The projection of the lookup-reduce: three exact terms of the pooled rows,
-// sums as accurate as plain fp32 ones (kChunkSums).
+// sums as accurate as plain fp32 ones (kChunkSums).  again: the tile's columns
+// [c, c + cnt) of a row that were stored from sums that are not finite.
 struct ProjSumOp : ProjOp {
     static constexpr bool kChunkSums = true;
     int sum_blocks;   // unsplit: K blocks an accumulator holds
     int acc_blocks;   // split: K blocks an accumulator of the first term holds
+    const __nv_bfloat16 *acc, *w_pt;   // [B][3][kd], [d_out][kd]
+    int kd;
+    __device__ void again(const Tile &t, int row, int c, int cnt) const {
+        const int o = t.m0 + row, n = t.n0 + c;
+        if (o >= d_out || n >= B) return;
+        sums_again(out + (int64_t)n * d_out + o, d_out, acc + (int64_t)n * 3 * kd, 3 * kd,
+                   w_pt + (int64_t)o * kd, 0, min(cnt, min(B, t.n0 + n_tile) - n), 1, kd, 1, kd);
+    }
 };
 template <int AR> struct ProjRowsSumOp : ProjRowsOp<AR> {
     static constexpr bool kChunkSums = true;
     int sum_blocks;   // K blocks an accumulator holds
+    const __nv_bfloat16 *acc, *w_pt;   // [B][3][kd], [d_out][kd]
+    int kd;
+    __device__ void again(const Tile &t, int row, int c, int cnt) const {
+        const int n = t.n0 + row, o = t.m0 + c;
+        if (n >= this->B || o >= this->d_out) return;
+        sums_again(this->out + (int64_t)n * this->d_out + o, 1, acc + (int64_t)n * 3 * kd, 0,
+                   w_pt + (int64_t)o * kd, kd, min(cnt, min(this->d_out, t.m0 + AR) - o), 1, kd,
+                   1, kd);
+    }
 };
 
 // The backward's dacc = W_p g (the projectors as stored, [E D_v][D'_v], are
@@ -1281,6 +1335,14 @@ struct DwMnSumOp : DwOp {
     static constexpr bool kChunkSums = true;
     static constexpr int kEpiWarps = 16;
     int sum_blocks;   // K blocks an accumulator holds
+    int B;
+    const __nv_bfloat16 *acc, *g;   // [B][3][N], [B][M]
+    __device__ void again(const Tile &t, int row, int c, int cnt) const {
+        const int o = t.m0 + row, n = t.n0 + c;
+        if (o >= M || n >= N) return;
+        sums_again(out + (int64_t)n * M + o, M, acc + n, 1, g + o, 0,
+                   min(cnt, min(N, t.n0 + n_tile) - n), 3 * (int64_t)N, N, M, B);
+    }
 };
 
 // dst[c][r] = src[r][c] for a rows x cols bf16 matrix (32 x 32 tiles), with
@@ -1468,6 +1530,7 @@ cudaError_t launch_dw_tc(const Dims &d, const CUtensorMap &g_t, const CUtensorMa
 
 template <int NSPLIT, class Op>
 static cudaError_t launch_dw_mn_op(const Dims &d, const CUtensorMap &g, const CUtensorMap &acc,
+                                   const __nv_bfloat16 *g_rows, const __nv_bfloat16 *acc_rows,
                                    float *dW, int *err, cudaStream_t st) {
     Op op;
     op.stamp = nullptr;
@@ -1491,6 +1554,9 @@ static cudaError_t launch_dw_mn_op(const Dims &d, const CUtensorMap &g, const CU
     dim3 grid(m_tiles, (op.N + op.n_tile - 1) / op.n_tile, 1);
     if constexpr (ChunkSums<Op>::value) {
         op.sum_blocks = 1;   // a tile's sums are few: the accuracy costs nothing
+        op.B = d.B;
+        op.acc = acc_rows;
+        op.g = g_rows;
         return launch_gemm_persistent<NSPLIT>(grid, g, g, acc, op, op.kb_total, d.pdl, st, 0);
     } else {
         op.stages = stages_for(NSPLIT, op.n_tile, op.kb_total);
@@ -1499,10 +1565,12 @@ static cudaError_t launch_dw_mn_op(const Dims &d, const CUtensorMap &g, const CU
                              g, acc, op, 0);
     }
 }
-cudaError_t launch_dw_mn(const Dims &d, const CUtensorMap &g, const CUtensorMap &acc, int terms,
-                         float *dW, int *err, cudaStream_t st) {
-    return terms == 3 ? launch_dw_mn_op<3, DwMnSumOp>(d, g, acc, dW, err, st)
-                      : launch_dw_mn_op<2, DwMnOp>(d, g, acc, dW, err, st);
+cudaError_t launch_dw_mn(const Dims &d, const CUtensorMap &g, const CUtensorMap &acc,
+                         const void *g_rows, const __nv_bfloat16 *acc_rows, int terms, float *dW,
+                         int *err, cudaStream_t st) {
+    const __nv_bfloat16 *gr = static_cast<const __nv_bfloat16 *>(g_rows);
+    return terms == 3 ? launch_dw_mn_op<3, DwMnSumOp>(d, g, acc, gr, acc_rows, dW, err, st)
+                      : launch_dw_mn_op<2, DwMnOp>(d, g, acc, gr, acc_rows, dW, err, st);
 }
 
 // tokens a tile of the dacc contraction: 128 where 256 would leave SMs idle
@@ -1657,7 +1725,12 @@ static cudaError_t launch_proj_rows(const Dims &d, const Ptrs &p, const TcMaps &
     op.kb_total = (d.E * d.d_v + kBlockK - 1) / kBlockK;
     op.out = static_cast<__nv_bfloat16 *>(p.out);
     op.vec = d.d_out % 8 == 0 && ((uintptr_t)p.out & 15) == 0;
-    if constexpr (ChunkSums<Op>::value) op.sum_blocks = sum_blocks_of(op.kb_total);
+    if constexpr (ChunkSums<Op>::value) {
+        op.sum_blocks = sum_blocks_of(op.kb_total);
+        op.acc = p.acc_bf;
+        op.w_pt = mp.w_pt_rows;
+        op.kd = d.E * d.d_v;
+    }
     dim3 grid((d.d_out + AR - 1) / AR, (d.B + kTileM - 1) / kTileM, 1);
     if constexpr (ChunkSums<Op>::value)
         return launch_gemm_persistent<NSPLIT>(grid, mp.w_pt, mp.w_pt, mp.acc, op, op.kb_total,
@@ -1695,6 +1768,9 @@ static cudaError_t launch_proj_op(const Dims &d, const Ptrs &p, const TcMaps &mp
         op.sum_blocks = sum_blocks_of(per);
         op.acc_blocks = (per + hi - 1) / hi;
         op.n_acc = 1 + (per + op.acc_blocks - 1) / op.acc_blocks;
+        op.acc = p.acc_bf;
+        op.w_pt = mp.w_pt_rows;
+        op.kd = d.E * d.d_v;
     }
     return launch_gemm<NSPLIT>(grid, mp.w_pt, mp.w_pt, mp.acc, op, per, d.pdl, st);
 }
