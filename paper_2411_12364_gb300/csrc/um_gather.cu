@@ -596,7 +596,8 @@ __global__ void __launch_bounds__(dot::kThreads) proj_kernel(Dims d, Ptrs p) {
     __shared__ dot::Stage<Acc, TPT, NP> st;
     const int Kd = d.E * d.d_v, split = blockIdx.z;
     const int chunk = (Kd + d.p_splits - 1) / d.p_splits;
-    const int o0 = blockIdx.x * S::TN, b0 = blockIdx.y * S::TM;
+    const int o_tiles = (d.d_out + S::TN - 1) / S::TN;
+    const int o0 = blockIdx.x % o_tiles * S::TN, b0 = blockIdx.x / o_tiles * S::TM;
     pdl_wait();
     stamp_begin(p.stamp);
     pdl_trigger();
@@ -779,7 +780,10 @@ cudaError_t launch_gather(const Dims &d, const Ptrs &p, cudaStream_t st) {
 template <typename T, int TPT, int NP>
 static cudaError_t launch_proj_t(const Dims &d, const Ptrs &p, cudaStream_t st) {
     using S = dot::Shape<TPT, NP>;
-    dim3 grid((d.d_out + S::TN - 1) / S::TN, (d.B + S::TM - 1) / S::TM, d.p_splits);
+    // tiles along x, outputs first (2^20 tokens are more tiles than y takes)
+    const int64_t tiles = (int64_t)((d.d_out + S::TN - 1) / S::TN) * ((d.B + S::TM - 1) / S::TM);
+    if (tiles > 0x7fffffff) return cudaErrorInvalidValue;
+    dim3 grid((unsigned)tiles, 1, d.p_splits);
     // a dependent launch is spread over the SMs (see spread_smem)
     constexpr auto k = proj_kernel<T, TPT, NP>;
     const size_t sm = d.pdl ? spread_smem(0, static_smem_of<k>(), ctas_of(grid)) : 0;

@@ -47,8 +47,8 @@ __global__ void __launch_bounds__(kThreads) query_kernel(Dims d, Ptrs p, int red
     stamp_begin(p.stamp);
     pdl_trigger();
     const int a = blockIdx.z / d.q_splits, split = blockIdx.z % d.q_splits;
-    const int HD = d.H * d.d_k;
-    const int o0 = blockIdx.x * S::TN, b0 = blockIdx.y * S::TM;
+    const int HD = d.H * d.d_k, o_tiles = (HD + S::TN - 1) / S::TN;
+    const int o0 = blockIdx.x % o_tiles * S::TN, b0 = blockIdx.x / o_tiles * S::TM;
     const int chunk = (d.d_in + d.q_splits - 1) / d.q_splits;
     dot::Operands<TX, T> o;
     o.A = static_cast<const TX *>(p.x);
@@ -184,7 +184,8 @@ template <typename T, typename TX, int TPT, int NP>
 cudaError_t launch_query_t(const Dims &d, const Ptrs &p, bool reduce, cudaStream_t st) {
     using S = dot::Shape<TPT, NP>;
     const int HD = d.H * d.d_k;
-    dim3 grid((HD + S::TN - 1) / S::TN, (d.B + S::TM - 1) / S::TM, d.A * d.q_splits);
+    // tiles along x, outputs first (2^20 tokens are more tiles than y takes)
+    dim3 grid(((HD + S::TN - 1) / S::TN) * ((d.B + S::TM - 1) / S::TM), 1, d.A * d.q_splits);
     const unsigned cl = reduce && d.q_splits > 1 ? (unsigned)d.q_splits : 1u;
     constexpr auto k = query_kernel<T, TX, TPT, NP>;
     const size_t sm = d.pdl ? spread_smem(0, static_smem_of<k>(), ctas_of(grid)) : 0;
