@@ -328,7 +328,10 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS) gather_bucket_kernel(
 // The same for fp32 rows, with compensated sums (Dot2).  VPL: 16-byte vectors
 // of a row that a lane owns (2: rows of up to 256 values; half as many rows in
 // flight).  A sum and its error term take twice the registers of a plain sum,
-// so half as many CTAs per SM.
+// so half as many CTAs per SM.  Dot2 has fp32's range: a sum that is not finite
+// (it may have passed FLT_MAX on the way) or so small that its products' error
+// terms may have underflowed is taken again in fp64.
+constexpr float kDot2Min = 0x1p-96f;   // products that lose error terms are below 2^-101
 template <int THREADS, int VPL>
 __global__ void __launch_bounds__(THREADS, 512 / THREADS) gather_bucket_exact(Dims d, Ptrs p) {
     using T = float;
@@ -413,7 +416,16 @@ __global__ void __launch_bounds__(THREADS, 512 / THREADS) gather_bucket_exact(Di
             o.c = v.y;
             all.merge(o);
         }
-        store_pooled<T>(d, p, b, i, all.value_any());
+        float sum = all.value_any();
+        if (!(fabsf(sum) >= kDot2Min && fabsf(sum) < INFINITY)) {
+            const float *col = static_cast<const float *>(p.values) + c;
+            const int ws = nc == 1 ? 0 : c / (Dv / nc);
+            double s = 0.0;
+            for (int j = start[qq]; j < start[qq] + tot[qq]; ++j)
+                s += (double)w_s[j * nc + ws] * (double)col[(int64_t)row_s[j] * Dv];
+            sum = (float)s;
+        }
+        store_pooled<T>(d, p, b, i, sum);
     }
     stamp_end(p.stamp);
 }
@@ -640,6 +652,12 @@ __global__ void proj_reduce_kernel(Dims d, Ptrs p) {
 #pragma unroll
             for (int sp = 0; sp < 8; ++sp) sum.two_sum_into(v[sp]);
             out = sum.value_any();
+            if (!(fabsf(out) < INFINITY)) {   // beyond fp32's range on the way, perhaps
+                double s = 0.0;
+#pragma unroll
+                for (int sp = 0; sp < 8; ++sp) s += (double)v[sp];
+                out = (float)s;
+            }
         } else {
             out = 0.f;
 #pragma unroll
