@@ -441,7 +441,11 @@ __global__ void __launch_bounds__(THREADS, 512 / THREADS) gather_bucket_exact(Di
 // a lookup of 2048 tokens at mid_4m 84.0 -> 79.1, prefill_16k 1902 -> 1888
 // (376 us for 2.2 GB, 5.9 TB/s); with component cores, whose weights are
 // another dependent read, it is slower (180 -> 186 us at mid_4m with 1000).
-// HALVES: the block's rows as two sums, of the first and the second half.
+// HALVES (E = 4): the block's rows as two sums, of the first and the second
+// half, which are the sums of the bucketed gather's two warps a block, bit for
+// bit.  Else (E = 9, 16, which took the general kernel's eight partial sums
+// before) 8 rows at a time by a tree: at most n / 8 + 5 roundings on the way to
+// a sum of n rows, no more than the n / 8 + 8 there.
 constexpr int kGWarps = 4;
 constexpr int kGSlots = 256;   // slots a token
 template <bool ADDR, bool HALVES>
@@ -515,12 +519,35 @@ __global__ void __launch_bounds__(32 * kGWarps, 32 / kGWarps) gather_warp_kernel
                     val[u] = (ok && active) ? ld_stream(V + (int64_t)row_s[j] * Dv)
                                             : make_uint4(0, 0, 0, 0);
                 }
+                if constexpr (HALVES) {
 #pragma unroll
-                for (int u = 0; u < kUnroll; ++u) {
-                    float f[EPV];
-                    unpack<__nv_bfloat16>(val[u], f);
+                    for (int u = 0; u < kUnroll; ++u) {
+                        float f[EPV];
+                        unpack<__nv_bfloat16>(val[u], f);
 #pragma unroll
-                    for (int c = 0; c < EPV; ++c) acc[c] = fmaf(wu[u], f[c], acc[c]);
+                        for (int c = 0; c < EPV; ++c) acc[c] = fmaf(wu[u], f[c], acc[c]);
+                    }
+                } else {   // the 8 rows by a tree
+                    static_assert(kUnroll == 8, "pairs, fours, eight");
+                    float four[EPV];
+#pragma unroll
+                    for (int u = 0; u < kUnroll; u += 4) {
+                        float f0[EPV], f1[EPV], two[EPV];
+                        unpack<__nv_bfloat16>(val[u], f0);
+                        unpack<__nv_bfloat16>(val[u + 1], f1);
+#pragma unroll
+                        for (int c = 0; c < EPV; ++c)
+                            two[c] = fmaf(wu[u + 1], f1[c], wu[u] * f0[c]);
+                        unpack<__nv_bfloat16>(val[u + 2], f0);
+                        unpack<__nv_bfloat16>(val[u + 3], f1);
+#pragma unroll
+                        for (int c = 0; c < EPV; ++c) {
+                            const float s4 =
+                                two[c] + fmaf(wu[u + 3], f1[c], wu[u + 2] * f0[c]);
+                            if (u == 0) four[c] = s4;
+                            else acc[c] += four[c] + s4;
+                        }
+                    }
                 }
             }
             if (HALVES && !part) {
