@@ -597,6 +597,8 @@ ultramem_status pool_and_project(ultramem_layer *L, const Dims &d0, Ptrs p,
     cudaError_t e;
     Dims d = d0;
     int n = 0;
+    // only the calls that reset the stamps first write them
+    auto staged = [&](int stage) { return slot_pos ? p : stage_ptrs(L, p, stage); };
     const int64_t macs = (int64_t)d.B * d.E * d.d_v * d.d_out;
     CUtensorMap acc_map;
     const bool tc = L->tc && d.has_proj && macs >= kTcLookupMacs &&
@@ -608,7 +610,7 @@ ultramem_status pool_and_project(ultramem_layer *L, const Dims &d0, Ptrs p,
     }
     bool gathered = false;
     if (tc && !slot_pos &&
-        (e = um::launch_gather_addresses(d, stage_ptrs(L, p, 3), &gathered, st)) != cudaSuccess)
+        (e = um::launch_gather_addresses(d, staged(3), &gathered, st)) != cudaSuccess)
         return from_cuda(e);
     if (gathered) {
         n = 1;
@@ -616,7 +618,7 @@ ultramem_status pool_and_project(ultramem_layer *L, const Dims &d0, Ptrs p,
         e = slot_pos ? um::launch_shard_slots(d, p, slot_pos, st)
                      : um::launch_slots_from_addresses(d, p, st);
         if (e != cudaSuccess) return from_cuda(e);
-        if ((e = um::launch_gather(d, stage_ptrs(L, p, 3), st)) != cudaSuccess)
+        if ((e = um::launch_gather(d, staged(3), st)) != cudaSuccess)
             return from_cuda(e);
         n = 2;
     }
@@ -624,11 +626,11 @@ ultramem_status pool_and_project(ultramem_layer *L, const Dims &d0, Ptrs p,
         um::TcMaps mp = L->maps;
         mp.acc = acc_map;
         d.pdl = 1;   // the projector's tiles stream in while the gather finishes
-        if ((e = um::launch_proj_tc(d, stage_ptrs(L, p, 4), mp, 3, st)) != cudaSuccess)
+        if ((e = um::launch_proj_tc(d, staged(4), mp, 3, st)) != cudaSuccess)
             return from_cuda(e);
         n += 1;
     } else if (d.has_proj) {
-        if ((e = um::launch_proj(d, stage_ptrs(L, p, 4), st)) != cudaSuccess)
+        if ((e = um::launch_proj(d, staged(4), st)) != cudaSuccess)
             return from_cuda(e);
         n += 2;
     }
