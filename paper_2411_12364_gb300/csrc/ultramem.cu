@@ -365,7 +365,7 @@ Ptrs make_ptrs(ultramem_layer *L) {
     p.tau = L->ws.tau;
     p.cand = reinterpret_cast<unsigned long long *>(L->ws.akey);
     p.sel_w = L->ws.sel_w;
-    p.acc = L->ws.acc;
+    p.acc = L->tc ? reinterpret_cast<float *>(L->ws.acc_bf) : L->ws.acc;
     p.proj_part = L->ws.proj_part;
     p.sel_row = L->ws.sel_row;
     p.sel_p = L->ws.sel_p;
@@ -800,7 +800,9 @@ ultramem_status ultramem_create(const ultramem_config *cfg, const ultramem_weigh
     if (e == cudaSuccess) e = dalloc(&ws.sel_w, hm * nc);
     if (e == cudaSuccess) e = dalloc(&ws.sel_row, hm);
     if (e == cudaSuccess) e = dalloc(&ws.sel_p, hm);
-    if (e == cudaSuccess) e = dalloc(&ws.acc, cfg->has_proj ? Bm * d.E * d.d_v : 1);
+    // (the tensor path's pooled rows, acc or acc_bf, share one array: no call
+    // uses both)
+    if (e == cudaSuccess && !L->tc) e = dalloc(&ws.acc, cfg->has_proj ? Bm * d.E * d.d_v : 1);
     if (e == cudaSuccess) e = dalloc(&ws.proj_part, cfg->has_proj ? pmax * d.d_out : 1);
     if (e == cudaSuccess) e = dalloc(&ws.core, (size_t)H * r * r);
     if (e == cudaSuccess && nc > 1) e = dalloc(&ws.cores, (size_t)H * nc * r * r);
@@ -1076,7 +1078,7 @@ ultramem_status ultramem_lookup_reduce_backward(ultramem_layer *L, const int64_t
                 return from_cuda(e);
             n += 6;
         } else {
-            if ((e = um::launch_backward_proj(d, L->ws.acc, g, dw_proj, st)) != cudaSuccess)
+            if ((e = um::launch_backward_proj(d, p.acc, g, dw_proj, st)) != cudaSuccess)
                 return from_cuda(e);
             n += 3;
         }
