@@ -1332,7 +1332,8 @@ __global__ void __launch_bounds__(kThreads, MINB) select_kernel(Dims d, Ptrs p) 
 // The scores, the order and so the selection are those of select_block, bit
 // for bit.  What a warp cannot hold (longer lists than kWCap or kWTop, scores
 // that are not finite, a list shorter than k) it leaves to select_block: its
-// CTA takes those (token, head)s one by one after its warps are done.
+// CTA takes those (token, head)s one by one after its warps are done (12 to 30 us
+// for a single one, n = 3000 with 384 tokens), but for zero queries.
 // About 7100 warp instructions a selection at prefill_16k.  Measured on GB300:
 // the selection of prefill_16k 1660 -> 620 us (a pass 2930 -> 1902), at mid_4m with
 // 1000 tokens and two cores 118 -> 64 us, at decode_1m with 2000 tokens (every
@@ -2106,6 +2107,79 @@ __device__ __forceinline__ bool select_warp(const Dims &d, const Ptrs &p, int bh
     return true;
 }
 
+// A (token, head) whose query is zero (a padding token: all its scores tie, which
+// overflows a warp's lists).  Every score that is a number is then zero, so by
+// address the slots are the first row with the first m <= k columns (of the axes'
+// candidates, or of all keys when each scores zero); false, nothing written,
+// where a factor that is not finite may make other ones.  One warp.  Retrievals
+// of zero tokens, a block per (token, head) -> the block's search for a CTA's
+// eight one by one -> this: decode_1m with 800 tokens 337 -> 619 -> 43 us, mid_4m
+// with 512 270 -> 615 -> 72, with 4096 4153 -> 5776 -> 1723 (the list passes, which
+// write every key).
+template <bool LISTS>
+__device__ __noinline__ bool select_zero_query(const Dims &d, const Ptrs &p, int bh, int *sel) {
+    const int lane = threadIdx.x & 31, m = d.m, K = d.K, G = d.n_segs;
+    const int b = bh / d.H, h = bh - b * d.H, HD = d.H * d.d_k;
+    bool nz = false;
+    for (int e = lane; e < 2 * d.d_k; e += 32) {
+        const int axis = e >= d.d_k, a = axis && d.A == 2;
+        nz = nz || p.q_part[((int64_t)a * d.B + b) * HD + h * d.d_k + e - axis * d.d_k] != 0.f;
+    }
+    if (__any_sync(kFull, nz)) return false;
+    const uint32_t zero = f2ord(0.f);
+    bool ok = true;
+    const int rr = d.r * d.r, ncrr = d.nc > 1 ? d.nc * rr : 0;
+    for (int e = lane; e < rr; e += 32) ok = ok && fabsf(p.core[(int64_t)h * rr + e]) < INFINITY;
+    for (int e = lane; e < ncrr; e += 32)
+        ok = ok && fabsf(p.cores[(int64_t)h * ncrr + e]) < INFINITY;
+    if (!__all_sync(kFull, ok)) return false;
+    for (int s = 0; s < 2; ++s) {
+        const int64_t li = (int64_t)bh * 2 + s;
+        const int need = s ? m : 1;   // positions of the axis that are used
+        int *at = sel + s * kWMaxK;
+        if constexpr (LISTS) {
+            const uint32_t *cnt = p.gstat + li * G;
+            const u64 *seg = p.cand + li * G * kSeg;
+            int c = 0;
+            for (int g = lane; g < G; g += 32) c += (int)min(__ldcg(cnt + g), (uint32_t)kSeg);
+            if ((int)__reduce_add_sync(kFull, c) < d.k) return false;
+            for (int g = 0, got = 0; got < need; ++g) {   // (ends: k >= need are listed)
+                const int n = (int)min(__ldcg(cnt + g), (uint32_t)kSeg);
+                for (int e = lane; e < n && got + e < need; e += 32) {
+                    const u64 x = __ldcg(seg + (int64_t)g * kSeg + e);
+                    at[got + e] = (int)pos_of(x);
+                    ok = ok && key_of(x) == zero;
+                }
+                got += n;
+            }
+        } else {
+            const uint4 *A = reinterpret_cast<const uint4 *>(p.akey + li * K);
+#pragma unroll 4
+            for (int i = lane; i < K >> 2; i += 32) {
+                const uint4 v = __ldcg(A + i);
+                ok = ok && v.x == zero && v.y == zero && v.z == zero && v.w == zero;
+            }
+            for (int e = lane; e < need; e += 32) at[e] = e;
+        }
+    }
+    if (!__all_sync(kFull, ok)) return false;
+    __syncwarp();
+    const uint32_t N = (uint32_t)d.N;
+    const float w = d.act == ULTRAMEM_ACT_SOFTMAX ? 1.f / (float)m : 0.f;
+    for (int e = lane; e < m; e += 32) {
+        const int64_t o = (int64_t)bh * m + e, v = (int64_t)sel[0] * K + sel[kWMaxK + e];
+        const uint32_t vs = (uint32_t)shuffle_address(d, p.perm, (uint64_t)v);   // Eq. 14
+        p.sel_p[o] = (int)(vs / N);
+        p.sel_row[o] = (int)(vs % N);
+        if (p.idx_out) p.idx_out[o] = v;
+        for (int ci = 0; ci < d.nc; ++ci) {
+            p.sel_w[o * d.nc + ci] = w;
+            if (p.w_out) p.w_out[o * d.nc + ci] = w;
+        }
+    }
+    return true;
+}
+
 // A (token, head) that its warp left to the block.
 template <int RM>
 __device__ __noinline__ void select_left(const Dims &d, const Ptrs &p, int bh,
@@ -2113,6 +2187,26 @@ __device__ __noinline__ void select_left(const Dims &d, const Ptrs &p, int bh,
     SelShared &sh = *reinterpret_cast<SelShared *>(smem);
     select_block<__nv_bfloat16, 4, (RM > 2 ? kMaxR : 2), false, false>(
         d, p, bh, smem + sizeof(SelShared), sh);
+}
+
+// The CTA's warps in `left`, without those of zero queries, which they settle.
+// Whole block.  (Out of line, and before the loop over the rest: the kernel's own
+// code then stays as fast; with the call inside the loop, or the loop inside it,
+// retrievals with lists took 1 to 2 % longer.)
+template <int RM, bool LISTS>
+__device__ __noinline__ unsigned select_zeros(const Dims &d, const Ptrs &p, unsigned left,
+                                              unsigned char *smem) {
+    __shared__ unsigned again;
+    const int warp = threadIdx.x >> 5;
+    if (threadIdx.x == 0) again = 0u;
+    __syncthreads();
+    if ((left >> warp & 1u) &&
+        !select_zero_query<LISTS>(d, p, (int)blockIdx.x * kWarps + warp,
+                                  reinterpret_cast<int *>(smem) + warp * 2 * kWMaxK) &&
+        (threadIdx.x & 31) == 0)
+        atomicOr(&again, 1u << warp);
+    __syncthreads();
+    return again;
 }
 
 template <int RM, bool PKM, bool LISTS>
@@ -2132,7 +2226,8 @@ __global__ void __launch_bounds__(kThreads, 4) select_warp_kernel(Dims d, Ptrs p
             atomicOr(&left, 1u << warp);
     }
     __syncthreads();
-    for (unsigned t = left; t; t &= t - 1u) {   // uniform
+    for (unsigned t = left ? select_zeros<RM, LISTS>(d, p, left, smem_raw) : 0u; t;
+         t &= t - 1u) {   // uniform
         select_left<RM>(d, p, (int)blockIdx.x * kWarps + __ffs(t) - 1, smem_raw);
         __syncthreads();
     }
