@@ -213,9 +213,12 @@ __device__ int pick_bin_from_bottom(const int *hist, int &need) {
 // The exact top m of the share's pairs into list (sh.count entries: m, or
 // fewer than the share holds never) by a radix select of the m-th largest
 // key over the scores, recomputed each pass, with one shared atomic per
-// distinct bin and warp.  Whole block; ends with a barrier.
+// distinct bin and warp.  `fixed` leading key bits (0 or 16) are known: no key
+// is above those of `prefix`, and m keys share them.  Whole block; ends with a
+// barrier.
 __device__ __noinline__ void radix_top_m(Grid gd, u64 *list, const uint16_t *map, int i0, int nr,
-                                         int K, int m, ExactShared &sh) {
+                                         int K, int m, uint32_t prefix, int fixed,
+                                         ExactShared &sh) {
     // the address of (row i, column j); map: the numbers of the rows kept, or null
     auto addr = [&](int i, int j) {
         return (uint32_t)(i0 + (map ? (int)map[i] : i)) * (uint32_t)K + (uint32_t)j;
@@ -227,12 +230,12 @@ __device__ __noinline__ void radix_top_m(Grid gd, u64 *list, const uint16_t *map
     const int di = kThreads / K, dj = kThreads % K;
     if (threadIdx.x == 0) {
         sh.count = 0;
-        sh.prefix = 0;
+        sh.prefix = prefix;
         sh.need = m;
     }
     __syncthreads();
     // the m-th largest key, 8 bits a pass
-    for (int shift = 24; shift >= 0; shift -= 8) {
+    for (int shift = 24 - fixed; shift >= 0; shift -= 8) {
         for (int e = threadIdx.x; e < 256; e += kThreads) sh.hist[e] = 0;
         __syncthreads();
         const uint32_t pre = sh.prefix;
@@ -800,6 +803,8 @@ __global__ void __launch_bounds__(kThreads, 1)
         }
     }
     const Grid gd{R, S, Rp, Sp, r, d.pkm};
+    uint32_t prefix = 0u;   // see radix_top_m
+    int fixed = 0;
     if (!general) {
         // 3. group maxima, and tau
         const PassShape ps(nr, K);
@@ -841,9 +846,17 @@ __global__ void __launch_bounds__(kThreads, 1)
         }
         __syncthreads();
         general = sh.count > list_n || sh.count < m;   // (fewer: never expected)
-        __syncthreads();
+        // tied scores: when no group's maximum is above tau in its leading 16
+        // bits, those are the m-th largest key's as well
+        bool above = tau == 0u;
+#pragma unroll
+        for (int q = 0; q < kParts; ++q) above = above || gk[q] >> 16 > tau >> 16;
+        if (!__syncthreads_or(above)) {
+            prefix = tau & 0xffff0000u;
+            fixed = 16;
+        }
     }
-    if (general) radix_top_m(gd, list, map, i0, nr, K, m, sh);
+    if (general) radix_top_m(gd, list, map, i0, nr, K, m, prefix, fixed, sh);
     const int n = min(sh.count, list_n);
     if (sh.count < m && threadIdx.x == 0) atomicOr(p.err, kErrInternal);   // never expected
 
