@@ -391,7 +391,10 @@ Dims dims_for(const ultramem_layer *L, int B) {
     // large_20m with 256, prefill_16k) 2-5 % shorter steps, below it (mid_4m
     // with 128-512 tokens, large_20m with 64 and 128, decode grids) 3-60 %
     // longer.  Mode 2 (the default) takes them from 3.5 tiles per SM on;
-    // modes 0 and 1 force every key or the lists.
+    // modes 0 and 1 force every key or the lists.  (Those figures are the block-wise
+    // selection's.  With the warp-wise one the lists are the shorter form from 1.7
+    // tiles per SM on: retrievals 69.7 -> 62.7 us at decode_1m with 1024 tokens, 92.2
+    // -> 83.6 with 2000, 62.1 -> 55.1 at mid_4m with 256; the line has not been moved.)
     const int64_t list_tiles = (int64_t)((d.K + 255) / 256) * ((B + 127) / 128) * 2 * d.H;
     const bool long_grid = 2 * list_tiles >= 7 * (int64_t)um::device_sm_count();
     d.cand = L->cand_ok && (L->cand_mode == 1 || (L->cand_mode == 2 && long_grid)) ? 1 : 0;
@@ -581,15 +584,16 @@ constexpr int kLongBackward = 512;   // tokens, see ultramem_lookup_reduce_backw
 // slot_pos[s] of p.values.
 //
 // Tensor layers project on the tensor cores, with the pooled rows as three
-// bf16 terms, which carry the fp32 sums exactly, so the output is as accurate
-// as the CUDA-core projection's.  That one was the bound: 500 of 563 us at
-// the 4M-slot layer with 2048 tokens.  Measured on GB300, a call as graph
-// replays, CUDA cores -> tensor cores with the gather reading the addresses:
-// mid_4m 33.2 -> 11.3 us at 1 token, 55.5 -> 13.3 at 128, 562 -> 69 at 2048,
-// 2071 -> 272 at 8192; decode_1m 20.5 -> 8.8 at 1 token, 26.8 -> 10.1 at 64.
-// It is faster down to the smallest layers (13.3 -> 7.2 us at 2^18 multiply-
-// adds); the line at 2^19 leaves those on the four launches (slots, gather,
-// projection, reduce) that ultramem_last_launches has always reported there.
+// bf16 terms, which carry the fp32 sums exactly, and sums that err less than the
+// CUDA-core projection's (kChunkSums in um_tc_gemm.cu).  That one was the bound:
+// 500 of 563 us at the 4M-slot layer with 2048 tokens.  Measured on GB300, a call
+// as graph replays, CUDA cores -> tensor cores with the gather reading the
+// addresses: mid_4m 33.2 -> 11.6 us at 1 token, 55.5 -> 14.1 at 128, 571 -> 73.6
+// at 2048, 2071 -> 271 at 8192; decode_1m 20.8 -> 9.4 at 1 token, 80 -> 17 at 500.
+// The line at 2^19 is not the crossover: from 2^15 to 2^18 multiply-adds the
+// tensor cores take 7.4 us against 11.0.  It leaves those on the four launches
+// (slots, gather, projection, reduce) that ultramem_last_launches has always
+// reported there.
 // fp32 storage keeps the CUDA-core projection (compensated sums).
 constexpr int64_t kTcLookupMacs = 1ll << 19;
 ultramem_status pool_and_project(ultramem_layer *L, const Dims &d0, Ptrs p,
@@ -1011,8 +1015,10 @@ ultramem_status ultramem_lookup_reduce_backward(ultramem_layer *L, const int64_t
     // the rows of both), and the kernels are programmatic dependents of one
     // another (g and the slots were complete before the first).  Measured on
     // GB300, decode_1m with 2048 tokens: 301 -> 256 us a call (137 of it zeroing
-    // dV); below 512 tokens the separate slots, transposes and plain launches
-    // stay.
+    // dV).  Below 512 tokens the separate slots, transposes and plain launches
+    // stay, and with them the counts that ultramem_last_launches has always
+    // reported there.  That is not the crossover (decode_1m, dV given: 44 us so
+    // and 23 chained at 128 tokens, 41 and 29 at 256, 53 and 36 at 504).
     bool chained = false;
     if (dw_proj && d.has_proj && L->tc && L->dacc_tc && B >= kLongBackward &&
         L->cfg.d_out % 8 == 0) {

@@ -37,7 +37,8 @@
 // Fewer (token, head) pairs than half the SMs are split into shares of rows,
 // a CTA each, so that about one CTA per SM runs: each leaves the exact top m
 // of its share, and a second kernel ranks the shares' winners.
-// Shared memory is 8 (K r + D_k) bytes plus 9 to 18 KB (K r <= 25600 fits).
+// Shared memory is 8 (K r + D_k) bytes plus 9 to 18 KB (K r <= 25600 fits) and,
+// where there is room for it, step 1's stage: 40 KB (bf16) or 72 KB (fp32).
 #include "um_internal.cuh"
 
 namespace um {
@@ -612,14 +613,10 @@ __global__ void __launch_bounds__(kThreads, 1)
     pdl_trigger();
 
     const int HD = d.H * D;
-    const int64_t split_stride = (int64_t)d.A * d.B * HD;
-    for (int e = threadIdx.x; e < 2 * D; e += kThreads) {   // summed over the D_i splits
+    for (int e = threadIdx.x; e < 2 * D; e += kThreads) {
         const int axis = e / D, c = e - axis * D;
         const int a = (axis == 1 && d.A == 2) ? 1 : 0;
-        const float *src = p.q_part + ((int64_t)a * d.B + b) * HD + h * D + c;
-        float q = 0.f;
-        for (int sp = 0; sp < d.q_splits; ++sp) q += src[sp * split_stride];
-        qv[e] = q;
+        qv[e] = p.q_part[((int64_t)a * d.B + b) * HD + h * D + c];
     }
     if (threadIdx.x < r * r) core[threadIdx.x] = p.core[(int64_t)h * r * r + threadIdx.x];
     if (threadIdx.x < 256) sh.hist[threadIdx.x] = 0;

@@ -174,7 +174,8 @@ __global__ void __launch_bounds__(kThreads) gather_reg_kernel(Dims d, Ptrs p) {
 constexpr int kBMaxE = 16;
 constexpr int kMaxCores = 8;   // MCS component cores per head
 
-// bytes of one accumulator of the layer's gather (fp64 for fp32 storage)
+// bytes of one accumulator of the layer's gather (fp32 storage: fp64, or the
+// two halves of a Dot2)
 size_t acc_bytes(const Dims &d) { return d.dtype == ULTRAMEM_F32 ? 8 : 4; }
 
 size_t bucket_smem_bytes(const Dims &d, int warps) {

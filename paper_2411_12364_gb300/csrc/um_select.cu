@@ -984,8 +984,8 @@ __device__ __forceinline__ void select_block(const Dims &d, const Ptrs &p, int b
         cl_arrive_relaxed();
     }
     // C of this head (a weight: read before the dependency wait) and the
-    // row/column query of this (token, head), summed over its D_i splits:
-    // loaded before the keys, stored after them
+    // row/column query of this (token, head): loaded before the keys, stored
+    // after them
     const float core_e = threadIdx.x < r * r ? p.core[(int64_t)h * r * r + threadIdx.x] : 0.f;
     // MCS component cores (nc r^2 <= 2 kThreads), stored once key1 is free
     const int ncrr = d.nc > 1 ? d.nc * r * r : 0;
@@ -1004,8 +1004,10 @@ __device__ __forceinline__ void select_block(const Dims &d, const Ptrs &p, int b
         const int a = (axis == 1 && d.A == 2) ? 1 : 0;
         return p.q_part + ((int64_t)a * d.B + b) * HD + h * d.d_k + c;
     };
-    // the split-K partials of q, summed in fp64 with fp32 storage (one
-    // rounding of the query the weights are computed from)
+    // (the query kernel has added up the D_i splits: one round of these loops.
+    // Without them the warp-wise kernels, which end in this code, came out
+    // slower: retrievals with lists 85.9 -> 87.5 us at K = 16000 with 256 tokens,
+    // 67.4 -> 68.3 at K = 9000 with 520.)
     auto q_of = [&](int e) {
         const float *src = q_src(e);
         if constexpr (std::is_same<T, float>::value) {
@@ -1334,8 +1336,8 @@ __global__ void __launch_bounds__(kThreads, MINB) select_kernel(Dims d, Ptrs p) 
 // that are not finite, a list shorter than k) it leaves to select_block: its
 // CTA takes those (token, head)s one by one after its warps are done (12 to 30 us
 // for a single one, n = 3000 with 384 tokens), but for zero queries.
-// About 7100 warp instructions a selection at prefill_16k.  Measured on GB300:
-// the selection of prefill_16k 1660 -> 620 us (a pass 2930 -> 1902), at mid_4m with
+// About 6200 warp instructions a selection at prefill_16k.  Measured on GB300:
+// the selection of prefill_16k 1660 -> 650 us (a pass 2930 -> 1902), at mid_4m with
 // 1000 tokens and two cores 118 -> 64 us, at decode_1m with 2000 tokens (every
 // key) 105 -> 59 us.  Bound by latency: 8 warps a scheduler (64 registers),
 // chains of shared-memory reads, shuffles and warp reductions.
@@ -2303,12 +2305,14 @@ size_t select_smem_bytes(const Dims &d) { return sel_offsets(d).total; }
 // (35 with every key), the blocks longer grids.  Measured on GB300, a
 // retrieval, blocks -> warps: with the lists 64.5 -> 69.9 us at 800 (mid_4m,
 // 200 tokens), 62.4 -> 65.8 and 80.7 -> 77.4 at 1024 (K = 4096 and 5000),
-// 103.0 -> 100.4 at 1600; with every key (K = 2048) 42.4 -> 49.2 at 1000,
-// 82.0 -> 69.2 at 2000.
+// 103.0 -> 100.4 at 1600 (the lists forced there; where the scoring takes them by
+// itself just over 1000 (1024, 1040 at K = 9000), K = 8600, 9000, 16000 and 16000 with 4, 2, 4 and 2 heads,
+// 79.8 -> 70.7, 74.3 -> 66.4, 91.5 -> 84.7 and 89.8 -> 82.5); with every key (K =
+// 2048) 42.4 -> 49.2 at 1000, 82.0 -> 69.2 at 2000.
 constexpr int64_t kWarpGridLists = 1000, kWarpGridKeys = 1500;
 static bool warp_select_fits(const Dims &d, const Ptrs &p) {
-    return d.dtype == ULTRAMEM_BF16 && d.q_splits == 1 && d.r <= 4 && d.k <= kWMaxK &&
-           d.m <= d.k && d.d_k <= kWMaxD && d.dk % 8 == 0 &&
+    return d.dtype == ULTRAMEM_BF16 && d.r <= 4 && d.k <= kWMaxK && d.m <= d.k &&
+           d.d_k <= kWMaxD && d.dk % 8 == 0 &&
            (((uintptr_t)p.k_row | (uintptr_t)p.k_col) & 15) == 0 &&
            (d.cand || (d.K % 4 == 0 && d.K >= 1024)) &&
            (int64_t)d.B * d.H > (d.cand ? kWarpGridLists : kWarpGridKeys);

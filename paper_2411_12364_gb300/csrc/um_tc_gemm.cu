@@ -131,7 +131,7 @@ constexpr uint32_t kMnBoxBytes = 64 * 128;   // 64 K rows of 64 bf16
 // thirds of them, and an accumulator holds few K blocks; the accumulators are
 // added up rounded.  Unsplit (persistent kernel): op.sum_blocks K blocks of 64
 // each, the epilogue warps keep the sums in registers (0.0003 and 0.0003; a
-// lookup of 2048 tokens at mid_4m 68.7 -> 73.4 us, 75 with one K block each).
+// lookup of 2048 tokens at mid_4m 68.7 -> 73.6 us, 75 with one K block each).
 // Split: the first term's blocks over all but one of the accumulators that
 // TMEM has room for (op.acc_blocks blocks each), the smaller terms of all
 // blocks in accumulator 0 (64 tokens at mid_4m: 0.00031, 0.00048 -> 0.00006;
@@ -1553,7 +1553,7 @@ static cudaError_t launch_dw_mn_op(const Dims &d, const CUtensorMap &g, const CU
     op.out = dW;
     dim3 grid(m_tiles, (op.N + op.n_tile - 1) / op.n_tile, 1);
     if constexpr (ChunkSums<Op>::value) {
-        op.sum_blocks = 1;   // a tile's sums are few: the accuracy costs nothing
+        op.sum_blocks = 1;   // dW_p is fp32: all of a sum's bits are seen
         op.B = d.B;
         op.acc = acc_rows;
         op.g = g_rows;
